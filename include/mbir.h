@@ -119,7 +119,9 @@ typedef struct {
 /* TAB mode normally also stores every A-scan's active pairs as records
  * grouped by first tap sample (the system matrix of Section 3) so that A x
  * and A^T stream them: 24 bytes per active pair for the CUDA-core kernels,
- * packed to 16 (FP32 form) or 12 bytes (BF16 form) for the tensor-core ones;
+ * packed to 16 (FP32 form) or 12 bytes (BF16 form) for the tensor-core ones,
+ * of which A x and A^T each hold a copy in their own order (without memory
+ * for the second copy A^T runs on the CUDA cores);
  * this flag keeps the on-the-fly record path of A x instead (less memory,
  * slower). */
 #define MBIR_FLAG_NO_RECORDS 1
@@ -176,8 +178,9 @@ typedef struct {
     int adjoint_tensor_cores;    /* 1 if A^T runs on the tensor cores (see MBIR_FLAG_NO_TENSOR_CORES) */
     int forward_tensor_cores;    /* 1 if A x runs on the tensor cores */
     int64_t n_records;           /* TAB records: active (pixel, A-scan) pairs held, else 0 */
-    int64_t record_bytes;        /* bytes of the record list as held: 24 per pair sorted (CUDA-core A x),
-                                  * 16 (FP32 form) or 12 (BF16 form) packed for the tensor cores */
+    int64_t record_bytes;        /* bytes of one record list as held: 24 per pair sorted (CUDA-core A x),
+                                  * 16 (FP32 form) or 12 (BF16 form) packed for the tensor cores (one list
+                                  * each for A x and A^T) */
     int tc_forward_variant;      /* tensor-core A x variant in use: 0 record loads through the L1, 1 records
                                   * past the L1 and the gathered image kept there */
     int tc_adjoint_variant;      /* tensor-core A^T variant in use: 0 four, 1 six records per thread and batch */

@@ -100,7 +100,8 @@ struct ReqDesc {
     int nblk;              // pixel blocks of kRedThreads
     // tensor-core A^T tables (tc != 0: the accumulators are allocated)
     int tc;
-    const int* tc_tile;
+    const int* tb_tile;
+    TbRecs tbrec;
     unsigned long long* tc_acc;   // this request's per-pixel fixed-point sums (zero between steps)
     float tc_bound;        // the geometry's scale bound of those sums
     // tensor-core A^T and A x of tc_stream.cuh (tcb, tcs != 0)
@@ -418,7 +419,7 @@ __global__ void __launch_bounds__(TbShape<BF16>::threads, 1) eng_bwd_tcs_kernel(
             if (!R.tc || !eng_pool_live(L.pool, rq, 1, nitems, flag)) continue;
             const void* tab = BF16 ? (const void*)R.tab_bf : (const void*)R.tab;
             const void* e = BF16 ? (const void*)R.ebf : (const void*)R.e;
-            const TbView V{R.P, R.tb4l, R.tb4_bop, tab, e, R.rec_off, R.tc_tile, R.tf4_crange, R.tkey, R.tw,
+            const TbView V{R.P, R.tb4l, R.tb4_bop, tab, e, R.rec_off, R.tb_tile, R.tf4_crange, R.tbrec,
                            R.tc_acc, reinterpret_cast<const unsigned int*>(L.pool + 3 * rq + 2), R.tc_bound,
                            L.pool + 3 * rq + 1};
             const bool ok = R.bvar ? tcs_adjoint_pool<BF16, 1>(V, smem, tmem, mphase, bphase, R.D.status)
@@ -775,7 +776,8 @@ void fill_desc(ReqDesc& d, const Request* r)
     d.sub = g->fwd_sub;
     d.nblk = r->nblk;
     d.tc = g->d_tb4_bop ? 1 : 0;
-    d.tc_tile = g->d_tc_tile;
+    d.tb_tile = g->d_tb_tile;
+    d.tbrec = TbRecs{g->d_tb_key, g->d_tb_w};
     d.tc_acc = r->acc;
     d.tc_bound = g->tc_bound;
     d.tcb = g->d_tb4_bop ? 1 : 0;

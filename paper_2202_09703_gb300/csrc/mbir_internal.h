@@ -397,6 +397,9 @@ struct mbir_geometry {
     float4* d_rec_w;
     uint2* d_tc_key;       // packed records: keys
     void* d_tc_w;          // and weights (uint2 in the FP32 form, uint32 in the BF16 form)
+    void* d_tb_key;        // the A^T's copy of the packed records, each tile's in pixel order (tc_apply.cuh)
+    uint32_t* d_tb_w;
+    int* d_tb_tile;        // its first record of every tile, from the A-scan's first: K x (tiles + 1)
     int2* d_runs;
     int fwd_sub;           // 32-sample spans per A x window (autotuned)
     double fwd_tune_ms[3]; // measured A x times of windows of 1, 2, 4 spans
@@ -406,7 +409,6 @@ struct mbir_geometry {
     float* h_tvert;        // host copy: vertical two-way time per image row (samples)
     int* d_win_counter;    // work counter of the A x launch
     // tensor-core A^T (see tc_adjoint.cu, tc_stream.cuh)
-    int* d_tc_tile;        // first record of every 128-sample tile, K x (tiles + 1)
     unsigned long long* w_tc_acc;   // per pixel: fixed-point sum, N + 1 (the last word: bits of max |e|)
     float tc_bound;        // scale bound of the fixed-point sums (build_tc_adjoint)
     int* d_tc_counter;

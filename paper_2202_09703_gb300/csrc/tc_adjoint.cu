@@ -1,5 +1,4 @@
-// Tables of the tensor-core A^T (tcs_adjoint_pool, tc_stream.cuh): the first
-// record of every tile, the per-pixel fixed-point accumulators and the bound
+// Tables of the tensor-core A^T (tcs_adjoint_pool, tc_stream.cuh): the per-pixel fixed-point accumulators and the bound
 // that sets their scale, the table operand, and the launch: max |e| of the
 // residual, the pool (one integer addition per record into its pixel's sum),
 // then the sums turned into FP32.  Integer addition is associative, so the
@@ -65,67 +64,42 @@ __global__ void tc_finish_kernel(int N, const unsigned long long* __restrict__ a
 }
 
 // *wmax = bits of the largest record weight w (the four bilinear corners are non-negative and sum to w)
-template <typename WT>
-__global__ void tc_wmax_kernel(const WT* __restrict__ rw, long long n, unsigned int* __restrict__ wmax)
+template <bool BF16>
+__global__ void tc_wmax_kernel(TbRecs rec, long long n, unsigned int* __restrict__ wmax)
 {
     unsigned int m = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        m = max(m, __float_as_uint(fabsf(tc_rec_w(rw[i]))));
+    {
+        TbRec<BF16> r;
+        r.load(rec, (size_t)i);
+        m = max(m, __float_as_uint(fabsf(r.weight())));
+    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0 && m) atomicMax(wmax, m);
 }
 
-// first record of every 128-sample tile of every A-scan (records grouped by tile, n0 ascending from tile to
-// tile)
-__global__ void tc_tile_off_kernel(GeomParams P, int ntile, const long long* __restrict__ rec_off,
-                                   const uint2* __restrict__ rkey, int* __restrict__ tile_off)
-{
-    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    if (i >= (long long)P.K * (ntile + 1)) return;
-    const int k = (int)(i / (ntile + 1)), t = (int)(i - (long long)k * (ntile + 1));
-    const long long base = rec_off[k];
-    int lo = 0, hi = (int)(rec_off[k + 1] - base);
-    const int target = t * kTsTile;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (tc_rec_n0(rkey[base + mid]) < target) lo = mid + 1;
-        else hi = mid;
-    }
-    tile_off[i] = lo;
-}
-
-// First record of every tile, the per-pixel accumulators (N sums and the max |e| word after them, zeroed)
-// and the bound of the fixed-point scale: K x the largest record weight w x (the largest table row sum
+// The per-pixel accumulators (N sums and the max |e| word after them, zeroed) and the bound of the fixed-point scale: K x the largest record weight w x (the largest table row sum
 // of |T| + the largest |T|, for the tau = t0 tap), doubled for the rounding of the products;
 // cudaErrorNotSupported keeps the CUDA-core adjoint.
 cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
 {
     const GeomParams& P = g->P;
-    if (!g->d_tc_key || g->n_records <= 0) return cudaErrorNotSupported;
+    if (!g->d_tb_key || g->n_records <= 0) return cudaErrorNotSupported;
     const int N = P.W * P.H;
-    const int ntile = (P.M + kTsTile - 1) / kTsTile;
-    int* d_tile = nullptr;
     unsigned long long* d_acc = nullptr;
     int* d_ctr = nullptr;
-    cudaError_t e = cudaMalloc((void**)&d_tile, sizeof(int) * (size_t)P.K * (ntile + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_acc, sizeof(unsigned long long) * ((size_t)N + 1));
+    cudaError_t e = cudaMalloc((void**)&d_acc, sizeof(unsigned long long) * ((size_t)N + 1));
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_ctr, sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(d_acc, 0, sizeof(unsigned long long) * ((size_t)N + 1), st);
-    if (e == cudaSuccess) {
-        const long long items = (long long)P.K * (ntile + 1);
-        tc_tile_off_kernel<<<(int)((items + 255) / 256), 256, 0, st>>>(P, ntile, g->d_rec_off, g->d_tc_key, d_tile);
-        e = cudaGetLastError();
-    }
     unsigned int wbits = 0;
     if (e == cudaSuccess) {
         unsigned int* d_wmax = reinterpret_cast<unsigned int*>(d_acc + N);
+        const TbRecs rec{g->d_tb_key, g->d_tb_w};
         if (P.precision == MBIR_PREC_BF16)
-            tc_wmax_kernel<<<std::max(1, g->n_sm * 8), 256, 0, st>>>(reinterpret_cast<const uint32_t*>(g->d_tc_w),
-                                                                     g->n_records, d_wmax);
+            tc_wmax_kernel<true><<<std::max(1, g->n_sm * 8), 256, 0, st>>>(rec, g->n_records, d_wmax);
         else
-            tc_wmax_kernel<<<std::max(1, g->n_sm * 8), 256, 0, st>>>(reinterpret_cast<const uint2*>(g->d_tc_w),
-                                                                     g->n_records, d_wmax);
+            tc_wmax_kernel<false><<<std::max(1, g->n_sm * 8), 256, 0, st>>>(rec, g->n_records, d_wmax);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&wbits, d_wmax, sizeof(wbits), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(d_wmax, 0, sizeof(unsigned long long), st);
@@ -148,26 +122,24 @@ cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
     const double bound = 2.0 * P.K * (double)wmax * (tsum + tmax);
     if (e == cudaSuccess && !(bound > 0.0 && bound < 1e30)) e = cudaErrorNotSupported;
     if (e != cudaSuccess) {
-        void* ptrs[] = {d_tile, d_acc, d_ctr};
+        void* ptrs[] = {d_acc, d_ctr};
         for (void* p : ptrs) cudaFree(p);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
     }
-    g->d_tc_tile = d_tile;
     g->w_tc_acc = d_acc;
     g->d_tc_counter = d_ctr;
     g->tc_bound = (float)bound;
-    g->bytes += sizeof(int) * ((size_t)P.K * (ntile + 1) + 1) + sizeof(unsigned long long) * ((size_t)N + 1);
+    g->bytes += sizeof(int) + sizeof(unsigned long long) * ((size_t)N + 1);
     return cudaSuccess;
 }
 
 // The tables above, freed when the tensor-core A^T is not used after all.
 void free_tc_adjoint(mbir_geometry* g)
 {
-    void* ptrs[] = {g->d_tc_tile, g->w_tc_acc, g->d_tc_counter};
+    void* ptrs[] = {g->w_tc_acc, g->d_tc_counter};
     for (void* p : ptrs)
         if (p) cudaFree(p);
-    g->d_tc_tile = nullptr;
     g->w_tc_acc = nullptr;
     g->d_tc_counter = nullptr;
 }
@@ -222,7 +194,7 @@ cudaError_t build_tc_adjoint_stream(mbir_geometry* g, cudaStream_t st)
 {
     (void)st;
     const GeomParams& P = g->P;
-    if (!g->d_tc_tile || !g->w_tc_acc || !g->d_tf4_crange || !g->d_tc_counter)
+    if (!g->d_tb_tile || !g->w_tc_acc || !g->d_tf4_crange || !g->d_tc_counter)
         return cudaErrorNotSupported;
     Tb4Layout L{};
     for (int kw : {256, 224, 192, 160, 128, 96, 64}) {
@@ -270,8 +242,8 @@ cudaError_t build_tc_adjoint_stream(mbir_geometry* g, cudaStream_t st)
     if (e == cudaSuccess) {
         const int N = P.W * P.H;
         const void* tab = P.precision == MBIR_PREC_BF16 ? (const void*)g->d_tab_bf16 : (const void*)g->d_tab;
-        const TbView V{P, L, d_b, tab, nullptr, g->d_rec_off, g->d_tc_tile, g->d_tf4_crange, g->d_tc_key,
-                       g->d_tc_w, g->w_tc_acc, reinterpret_cast<const unsigned int*>(g->w_tc_acc + N),
+        const TbView V{P, L, d_b, tab, nullptr, g->d_rec_off, g->d_tb_tile, g->d_tf4_crange,
+                       TbRecs{g->d_tb_key, g->d_tb_w}, g->w_tc_acc, reinterpret_cast<const unsigned int*>(g->w_tc_acc + N),
                        g->tc_bound, g->d_tc_counter};
         e = cudaMalloc((void**)&d_view, sizeof(TbView));
         if (e == cudaSuccess) e = cudaMemcpy(d_view, &V, sizeof(TbView), cudaMemcpyHostToDevice);

@@ -70,6 +70,83 @@ __device__ __forceinline__ void tc_pack_w(const Pair& pr, uint32_t& w)
     w = w16 | (__float2uint_rn(pr.psi * 32768.0f) << 16);
 }
 
+// Records of the A^T, a copy of the same pairs with each tile's records in pixel order (tb_pack_kernel):
+//   key.x = pixel (bits 0-19) | table row (bits 20-30)
+//   key.y = n0 within its 128-sample tile (bits 25-31) | tau = t0 flag (bit 24) | fa x 2^23 (bits 0-22)
+// and, in the FP32 form in the same uint4, {w, 1 + psi}; in the BF16 form in an array of their own, uint32
+// {w16 | psi x 2^15 << 16} as above.  The fractions are kept as the mantissa of 1 + fraction.
+constexpr int kTbN0Shift = 25;
+constexpr uint32_t kTbFlag0 = 1u << 24;
+
+// The record arrays of a storage form, and one record of them.
+struct TbRecs {
+    const void* key;         // FP32 form: uint4 records; BF16 form: uint2 keys
+    const uint32_t* w;       // BF16 form: weights
+};
+
+template <bool BF16>
+struct TbRec {
+    uint2 key;
+    uint2 w;                 // BF16 form: w.x only
+
+    __device__ __forceinline__ int pixel() const { return (int)(key.x & kTcPixelMask); }
+    __device__ __forceinline__ int row() const { return (int)(key.x >> kTcRowShift); }
+    __device__ __forceinline__ int n0() const { return (int)(key.y >> kTbN0Shift); }      // within the tile
+    __device__ __forceinline__ bool flag0() const { return (key.y & kTbFlag0) != 0; }
+    __device__ __forceinline__ float fa1() const                                          // 1 + fa
+    {
+        return __uint_as_float((key.y & 0x7fffffu) | 0x3f800000u);
+    }
+    __device__ __forceinline__ float weight() const
+    {
+        if constexpr (BF16) return __uint_as_float(((w.x & 0xffffu) << 13) + 0x20000000u);
+        else return __uint_as_float(w.x);
+    }
+    __device__ __forceinline__ float psi1() const                                         // 1 + psi
+    {
+        if constexpr (BF16) return __uint_as_float(0x3f800000u + ((w.x >> 16) << 8));
+        else return __uint_as_float(w.y);
+    }
+    // record i of the arrays (read once: the loads bypass the L1)
+    __device__ __forceinline__ void load(const TbRecs& a, size_t i)
+    {
+        if constexpr (BF16) {
+            key = ldg_stream(reinterpret_cast<const uint2*>(a.key) + i);
+            w = make_uint2(ldg_stream(a.w + i), 0u);
+        } else {
+            const uint4 v = ldg_stream(reinterpret_cast<const uint4*>(a.key) + i);
+            key = make_uint2(v.x, v.y);
+            w = make_uint2(v.z, v.w);
+        }
+    }
+    __device__ __forceinline__ void store(uint2* keys, uint32_t* ws, size_t i) const
+    {
+        if constexpr (BF16) {
+            keys[i] = key;
+            ws[i] = w.x;
+        } else {
+            reinterpret_cast<uint4*>(keys)[i] = make_uint4(key.x, key.y, w.x, w.y);
+        }
+    }
+    // the record of pixel v from its pair; n0r: n0 less its tile's start
+    __device__ __forceinline__ void pack(int v, int trow, int n0r, const Pair& pr)
+    {
+        const uint32_t qa = min((uint32_t)__float2uint_rn(pr.w0 * 8388608.0f), 0x7fffffu);
+        key = make_uint2((uint32_t)v | ((uint32_t)trow << kTcRowShift),
+                         ((uint32_t)n0r << kTbN0Shift) | (pr.flag0 ? kTbFlag0 : 0u) | qa);
+        if constexpr (BF16) {
+            // round to 10 mantissa bits (a carry moves into the exponent), then rebase the exponent at 2^-63
+            const uint32_t u = __float_as_uint(pr.w) + 0x1000u;
+            const uint32_t w16 = pr.w >= 0x1p-63f ? min((u >> 13) - (64u << 10), 0xffffu) : 0u;
+            w = make_uint2(w16 | (__float2uint_rn(pr.psi * 32768.0f) << 16), 0u);
+        } else {
+            w = make_uint2(__float_as_uint(pr.w), __float_as_uint(1.0f + pr.psi));
+        }
+    }
+};
+template <bool BF16>
+__host__ __device__ constexpr size_t tb_key_bytes() { return BF16 ? sizeof(uint2) : sizeof(uint4); }
+
 // Shared-memory header of the tensor-core kernels: offset 0 the MMA mbarrier, 8 the tensor-memory address,
 // 16 the item slot, 20 the abort flag, 32 the table-copy mbarrier.
 __device__ __forceinline__ void tc_header_init(unsigned char* smem, uint32_t ncols)
@@ -95,16 +172,13 @@ __device__ __forceinline__ void tc_header_release(unsigned char* smem, uint32_t 
     if ((threadIdx.x >> 5) == 0) tmem_dealloc(tmem, ncols);
 }
 
-// Two values into packed FP16 high and low parts: hi = x rounded to 11 significant bits by Veltkamp's
-// splitting, (x (2^13 + 1)) - ((x (2^13 + 1)) - x) (exact in FP16 for |x| in [2^-14, 2^15]), and
-// lo = x - hi (exact in FP32) rounded to FP16; x = hi + lo to 2^-23 relative.  No packed conversion
-// is spent on the high part's remainder.
+// Two values into packed FP16 high and low parts: hi = x rounded to 11 significant bits (exact in FP16 for
+// |x| in [2^-14, 2^15]) and lo = x - hi (exact in FP32) rounded to FP16; x = hi + lo to 2^-23 relative.
 __device__ __forceinline__ void split2h_pair(float x0, float x1, uint32_t& hi, uint32_t& lo)
 {
-    const float t0 = __fmul_rn(x0, 8193.0f), t1 = __fmul_rn(x1, 8193.0f);
-    const float h0 = __fsub_rn(t0, __fsub_rn(t0, x0)), h1 = __fsub_rn(t1, __fsub_rn(t1, x1));
-    const __half2 H = __floats2half2_rn(h0, h1);
-    const __half2 L = __floats2half2_rn(__fsub_rn(x0, h0), __fsub_rn(x1, h1));
+    const __half2 H = __floats2half2_rn(x0, x1);
+    const float2 h = __half22float2(H);
+    const __half2 L = __floats2half2_rn(__fsub_rn(x0, h.x), __fsub_rn(x1, h.y));
     hi = *reinterpret_cast<const uint32_t*>(&H);
     lo = *reinterpret_cast<const uint32_t*>(&L);
 }

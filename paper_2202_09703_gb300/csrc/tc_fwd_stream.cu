@@ -211,6 +211,83 @@ __global__ void ts_batch_flag_kernel(GeomParams P, int R, int nparts, const long
     }
 }
 
+// The records of the A^T, every tile's in pixel order.  The A^T is bound by its per-pixel reductions in the L2,
+// which takes a sector (four pixels' sums) per reduction: 206 G/s where every lane meets another sector, 330,
+// 505 and 630 G/s for runs of 2, 4 and 8 neighbouring pixels.  In the A x's order (by n0, for its sums) the 32
+// records of a warp fell into 28 sectors; the pixels of one image row that a tile reaches lie side by side
+// (64 columns where the delay grows by two samples per column), so in pixel order they fall into about nine.
+// 512x1024 A^T: FP32 7.55 -> 5.83 ms; 256x512 0.478 -> 0.418 ms; 203x331 BF16 0.144 -> 0.128 ms.  It costs a
+// second copy of the packed records.
+// Block per (A-scan, tile): a bitmap of the tile's pixels, from which each record's place is counted.
+__host__ __device__ inline int tb_map_words(const GeomParams& P) { return ((P.W * P.H + 127) >> 7) << 2; }
+template <bool BF16>
+__global__ void __launch_bounds__(512)
+    tb_pack_kernel(GeomParams P, DevPtrs D, const long long* __restrict__ rec_off, const int* __restrict__ n0_off,
+                   const int2* __restrict__ skey, uint2* __restrict__ key, uint32_t* __restrict__ w)
+{
+    extern __shared__ uint32_t s_map[];                // a bit per pixel, then the exclusive sums of every four words
+    __shared__ int s_warp[16];
+    const int nword = tb_map_words(P);
+    int* s_sum = reinterpret_cast<int*>(s_map + nword);
+    const int ntile = (P.M + kTsTile - 1) / kTsTile;
+    const int k = (int)(blockIdx.x / ntile), t = (int)(blockIdx.x % ntile);
+    const int* no = n0_off + (size_t)k * (P.M + 1);
+    const int r0 = no[min(t * kTsTile, P.M)], r1 = no[min((t + 1) * kTsTile, P.M)];
+    if (r0 == r1) return;
+    const long long base = rec_off[k];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, R = P.Q + 1;
+    for (int i = tid; i < nword; i += blockDim.x) s_map[i] = 0u;
+    __syncthreads();
+    for (int r = r0 + tid; r < r1; r += blockDim.x) {
+        const int v = skey[base + r].x & kRecPixel;
+        atomicOr(s_map + (v >> 5), 1u << (v & 31));
+    }
+    __syncthreads();
+    const int per = 4 * ((nword / 4 + (int)blockDim.x - 1) / (int)blockDim.x), w0 = min(tid * per, nword),
+              w1 = min(w0 + per, nword);
+    int s = 0;
+    for (int i = w0; i < w1; ++i) s += __popc(s_map[i]);
+    int incl = s;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    int acc = incl - s;
+    for (int i = 0; i < warp; ++i) acc += s_warp[i];
+    for (int i = w0; i < w1; i += 4) {
+        s_sum[i >> 2] = acc;
+        acc += __popc(s_map[i]) + __popc(s_map[i + 1]) + __popc(s_map[i + 2]) + __popc(s_map[i + 3]);
+    }
+    __syncthreads();
+    for (int r = r0 + tid; r < r1; r += blockDim.x) {
+        const int v = skey[base + r].x & kRecPixel;
+        int at = r0 + s_sum[v >> 7] + __popc(s_map[v >> 5] & ((1u << (v & 31)) - 1u));
+        for (int i = (v >> 7) << 2; i < (v >> 5); ++i) at += __popc(s_map[i]);
+        Pair pr;
+        TbRec<BF16> rc;
+        if (tab_pair(P, D, k, v, pr)) {
+            rc.pack(v, pr.gi * R + pr.r, pr.n0 - t * kTsTile, pr);
+        } else {
+            rc.key = make_uint2((uint32_t)v, 0u);       // (not reached) a zero-weight record
+            rc.w = make_uint2(0u, 0x3f800000u);
+        }
+        rc.store(key, w, (size_t)(base + at));
+    }
+}
+
+// first record of every tile, from the A-scan's first
+__global__ void tb_tile_kernel(GeomParams P, const int* __restrict__ n0_off, int* __restrict__ tile_off)
+{
+    const int ntile = (P.M + kTsTile - 1) / kTsTile;
+    const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (i >= (long long)P.K * (ntile + 1)) return;
+    const int k = (int)(i / (ntile + 1)), t = (int)(i - (long long)k * (ntile + 1));
+    tile_off[i] = n0_off[(size_t)k * (P.M + 1) + min(t * kTsTile, P.M)];
+}
+
 // Tables of the tensor-core A x for a geometry with records: the A-scan order, the per-tile column ranges and
 // warp parts (from the first record of every n0), the table operand (FP32 form: two FP16 parts of the table scaled by
 // 2^texp; BF16 form: the BF16 table); cudaErrorNotSupported keeps the CUDA-core A x.
@@ -327,6 +404,37 @@ cudaError_t build_tc_forward_stream(mbir_geometry* g, cudaStream_t st)
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
+    // the A^T's copy of the records, where there is memory for it (else the CUDA-core A^T is kept)
+    void* d_tkey = nullptr;
+    uint32_t* d_tpw = nullptr;
+    int* d_toff = nullptr;
+    const size_t tksz = bf ? tb_key_bytes<true>() : tb_key_bytes<false>();
+    if (e == cudaSuccess) {
+        cudaError_t m = cudaMalloc((void**)&d_toff, sizeof(int) * (size_t)P.K * (ntile + 1));
+        if (m == cudaSuccess) m = cudaMalloc(&d_tkey, tksz * nrec);
+        if (m == cudaSuccess && bf) m = cudaMalloc((void**)&d_tpw, sizeof(uint32_t) * nrec);
+        if (m != cudaSuccess) {
+            cudaGetLastError();
+            cudaFree(d_toff);
+            cudaFree(d_tkey);
+            d_toff = nullptr;
+            d_tkey = nullptr;
+            if (m != cudaErrorMemoryAllocation) e = m;
+        }
+    }
+    if (e == cudaSuccess && d_tkey) {
+        auto kern = bf ? tb_pack_kernel<true> : tb_pack_kernel<false>;
+        const size_t sm = (size_t)tb_map_words(P) * 5;
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        if (e == cudaSuccess) {
+            const long long nt = (long long)P.K * (ntile + 1);
+            tb_tile_kernel<<<(int)((nt + 255) / 256), 256, 0, st>>>(P, d_n0, d_toff);
+            kern<<<P.K * ntile, 512, sm, st>>>(P, dev_ptrs(g), g->d_rec_off, d_n0, g->d_rec_key,
+                                              reinterpret_cast<uint2*>(d_tkey), d_tpw);
+            e = cudaGetLastError();
+        }
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    }
     // the kernel's view without the per-call fields
     TsView* d_view = nullptr;
     if (e == cudaSuccess) {
@@ -336,7 +444,7 @@ cudaError_t build_tc_forward_stream(mbir_geometry* g, cudaStream_t st)
         if (e == cudaSuccess) e = cudaMemcpy(d_view, &V, sizeof(TsView), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
-        void* ptrs[] = {d_n0, d_ord, d_ctr, d_cr, d_sp, d_b, d_view, d_key, d_pw};
+        void* ptrs[] = {d_n0, d_ord, d_ctr, d_cr, d_sp, d_b, d_view, d_key, d_pw, d_toff, d_tkey, d_tpw};
         for (void* p : ptrs) cudaFree(p);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
@@ -350,6 +458,10 @@ cudaError_t build_tc_forward_stream(mbir_geometry* g, cudaStream_t st)
     g->bytes += (sizeof(uint2) + wsz) * nrec;
     g->d_tc_key = d_key;
     g->d_tc_w = d_pw;
+    g->d_tb_key = d_tkey;
+    g->d_tb_w = d_tpw;
+    g->d_tb_tile = d_toff;
+    if (d_tkey) g->bytes += (tksz + (bf ? sizeof(uint32_t) : 0)) * nrec + sizeof(int) * (size_t)P.K * (ntile + 1);
     cudaFree(d_n0);
     g->d_tf_view = d_view;
     g->tf4 = L;

@@ -471,15 +471,17 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
             }
             tc_fence_before();
             __syncthreads();
-            if (tid == 0) {
+            if (tid == 32 * (kTsWarps - 1)) {
                 tc_fence_after();
-                const uint32_t b0 = smem_u32(sB) + (uint32_t)(c_lo / 8) * 128;
-                for (int s = 0; s < kw / 16; ++s) {
-                    umma_f16_ta(tD, tA + 8 * s, umma_desc(b0 + 256 * s, 128, sboB), idesc, s > 0);
+                // (one thread issues dozens of products: the descriptors are stepped, not rebuilt)
+                uint64_t db = umma_desc(smem_u32(sB) + (uint32_t)(c_lo / 8) * 128, 128, sboB);
+#pragma unroll 1
+                for (int s = 0; s < kw / 16; ++s, db += 256 >> 4) {
+                    umma_f16_ta(tD, tA + 8 * s, db, idesc, s > 0);
                     if (!BF16) {
                         // hi x lo, lo x hi
-                        umma_f16_ta(tD, tA + 8 * s, umma_desc(b0 + bpart + 256 * s, 128, sboB), idesc, true);
-                        umma_f16_ta(tD, tA + KA + 8 * s, umma_desc(b0 + 256 * s, 128, sboB), idesc, true);
+                        umma_f16_ta(tD, tA + 8 * s, db + (bpart >> 4), idesc, true);
+                        umma_f16_ta(tD, tA + KA + 8 * s, db, idesc, true);
                     }
                 }
                 umma_commit(smem_u32(smem));
@@ -503,7 +505,7 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
 // is one matrix product of the residual's Hankel tile H[n][m] = e[ts + 1 + n + m]
 // (128 x taps, in tensor memory as the A operand) and the table rows the tile's
 // records reach (one column range, the B operand resident in shared memory);
-// each record then combines four values of C with its bilinear weights (less
+// each record (a tile's are stored in pixel order, tb_pack_kernel) then combines four values of C with its bilinear weights (less
 // the tau = t0 tap of flagged records) into one contribution v and adds it to
 // its pixel's 64-bit fixed-point accumulator: round(v 2^s) by an integer atomic
 // (one scale 2^s per apply, tc_fixed_exponent), so the sum is exact and its
@@ -522,8 +524,7 @@ struct TbView {
     const long long* rec_off;
     const int* tile_off;         // first record of every tile, K x (ntile + 1)
     const uint32_t* crange;      // per (A-scan, tile): c_lo | c_hi << 16
-    const uint2* rkey;           // packed records (tc_apply.cuh): keys
-    const void* rw;              // and weights, uint2 (FP32 form) or uint32 (BF16 form)
+    TbRecs rec;                  // packed records, each tile's in pixel order (tc_apply.cuh)
     unsigned long long* acc;     // per pixel: the fixed-point sum (zero on entry)
     const unsigned int* emax;    // bits of max |e| over the residual (tc_emax)
     float bound;                 // K x max record weight x (max table row sum of |T| + max |T|), doubled
@@ -554,23 +555,13 @@ __device__ __forceinline__ float tcs_finish_pixel(unsigned long long a, unsigned
 }
 
 // A batch of records held in registers: records rb + u * NT + tid, u < U (NT threads per CTA).
-template <int U, typename WT>
-struct TbBatch {
-    uint2 key[U];
-    WT w[U];
-};
-
-template <int NT, int U, typename WT>
-__device__ __forceinline__ void tb_load(TbBatch<U, WT>& b, const uint2* __restrict__ rkey, const WT* __restrict__ rw,
-                                        long long base, int rb, int r1, int tid)
+template <int NT, int U, bool BF16>
+__device__ __forceinline__ void tb_load(TbRec<BF16> (&b)[U], const TbRecs& rec, long long base, int rb, int r1, int tid)
 {
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         const int r = rb + u * NT + tid;
-        if (r < r1) {
-            b.key[u] = __ldg(rkey + base + r);
-            b.w[u] = __ldg(rw + base + r);
-        }
+        if (r < r1) b[u].load(rec, (size_t)(base + r));
     }
 }
 
@@ -591,11 +582,8 @@ __device__ __forceinline__ bool tcs_adjoint_pool(const TbView& V, unsigned char*
     unsigned char* sB = smem + T.off_b;
     float* sC = reinterpret_cast<float*>(smem + T.off_c);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    using WT = typename TcW<BF16>::type;
     const int R = T.R, S = table_stride(P.Tw4);
     const int dR = P.G > 1 ? R : 0;                    // columns from a table row to the next plane's
-    const uint2* __restrict__ rkey = V.rkey;
-    const WT* __restrict__ rw = reinterpret_cast<const WT*>(V.rw);
     unsigned long long* __restrict__ acc = V.acc;
     const float fsc = ts_pow2(tc_fixed_exponent(*V.emax, V.bound));
     const uint32_t tA = tmem, tD = tmem + 128;
@@ -665,12 +653,13 @@ __device__ __forceinline__ bool tcs_adjoint_pool(const TbView& V, unsigned char*
         const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
         tc_fence_after();
         const uint32_t idesc = BF16 ? umma_idesc_bf16(kTsTile, kw) : umma_idesc_f16(kTsTile, kw);
-        const uint32_t b0 = smem_u32(sB) + (uint32_t)(c_lo / 8) * sboB;
-        for (int s = 0; s < T.ntap / 16; ++s) {
-            umma_f16_ta(tD, tA + 8 * s, umma_desc(b0 + 256 * s, 128, sboB), idesc, s > 0);
+        uint64_t db = umma_desc(smem_u32(sB) + (uint32_t)(c_lo / 8) * sboB, 128, sboB);
+#pragma unroll 1
+        for (int s = 0; s < T.ntap / 16; ++s, db += 256 >> 4) {
+            umma_f16_ta(tD, tA + 8 * s, db, idesc, s > 0);
             if (!BF16) {
-                umma_f16_ta(tD, tA + 8 * s, umma_desc(b0 + bpart + 256 * s, 128, sboB), idesc, true);
-                umma_f16_ta(tD, tA + HA + 8 * s, umma_desc(b0 + 256 * s, 128, sboB), idesc, true);
+                umma_f16_ta(tD, tA + 8 * s, db + (bpart >> 4), idesc, true);
+                umma_f16_ta(tD, tA + HA + 8 * s, db, idesc, true);
             }
         }
         umma_commit(smem_u32(smem));
@@ -689,15 +678,15 @@ __device__ __forceinline__ bool tcs_adjoint_pool(const TbView& V, unsigned char*
     tc_fence_before();
     __syncthreads();
     int nxt = *next;
-    if (tid == 0 && live_cur) issue_mma(cur);
+    if (tid == NTB - 32 && live_cur) issue_mma(cur);
     while (!*abort_flag) {
         const int kc = cur / ntile, tc = cur - kc * ntile;
         const long long base = __ldg(V.rec_off + kc);
         const int r0 = __ldg(V.tile_off + (size_t)kc * (ntile + 1) + tc);
         const int r1 = __ldg(V.tile_off + (size_t)kc * (ntile + 1) + tc + 1);
         // the first records of this item and the next item's window load during the products
-        TbBatch<U, WT> ba, bb;
-        tb_load<NTB>(ba, rkey, rw, base, r0, r1, tid);
+        TbRec<BF16> ba[U], bb[U];
+        tb_load<NTB, U>(ba, V.rec, base, r0, r1, tid);
         const float ew = nxt < nitems ? load_e(nxt) : 0.0f;
         float* sEc = sE0 + cbuf * T.ewin;
         float* sEn = sE0 + (cbuf ^ 1) * T.ewin;
@@ -732,26 +721,25 @@ __device__ __forceinline__ bool tcs_adjoint_pool(const TbView& V, unsigned char*
         tc_fence_before();
         __syncthreads();                                  // H of the next item in tensor memory
         const int nn = *next;
-        if (tid == 0 && live_nxt) issue_mma(nxt);
+        if (tid == NTB - 32 && live_nxt) issue_mma(nxt);
         // ---- the current item's records: four values of C each, one fixed-point addition per record; the
         // next batch loads while one is combined
         if (live_cur) {
-            const int ts = tc * kTsTile;
             const float* Cb = sC - c_lo;
-            auto run = [&](const TbBatch<U, WT>& bt, int rb) {
+            auto run = [&](const TbRec<BF16> (&bt)[U], int rb) {
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
                     const int r = rb + u * NTB + tid;
                     if (r >= r1) continue;
-                    const uint2 kk = bt.key[u];
-                    const int n0r = tc_rec_n0(kk) - ts, trow = tc_rec_row(kk);
+                    const TbRec<BF16>& rc = bt[u];
+                    const int n0r = rc.n0(), trow = rc.row();
                     const float* cr = Cb + n0r * T.cstride;
-                    const float fa = tc_rec_fa(kk), psi = tc_rec_psi(bt.w[u]);
+                    const float fa = rc.fa1() - 1.0f, psi = rc.psi1() - 1.0f;
                     // bilinear in the attenuation plane (psi), then in the phase (fa)
                     const float c00 = cr[trow], c10 = cr[trow + dR], c01 = cr[trow + 1], c11 = cr[trow + dR + 1];
                     const float a0 = fmaf(psi, c10 - c00, c00), a1 = fmaf(psi, c11 - c01, c01);
                     float v = fmaf(fa, a0 - a1, a1);
-                    if (kk.y & kTcFlag0) {
+                    if (rc.flag0()) {
                         // tau = t0 exactly: the last tap of the upper phase row lies outside the window
                         const size_t ti = (size_t)(trow + 1) * S + P.Tw - 1;
                         float2 tl;
@@ -759,16 +747,16 @@ __device__ __forceinline__ bool tcs_adjoint_pool(const TbView& V, unsigned char*
                         else tl = __ldg(reinterpret_cast<const float2*>(V.tab) + ti);
                         v -= (1.0f - fa) * fmaf(psi, tl.y - tl.x, tl.x) * sEc[n0r + P.Tw - 1];
                     }
-                    v *= tc_rec_w(bt.w[u]);
-                    red_add_global_u64(acc + (kk.x & kTcPixelMask), (unsigned long long)__float2ll_rn(v * fsc));
+                    v *= rc.weight();
+                    red_add_global_u64(acc + rc.pixel(), (unsigned long long)__float2ll_rn(v * fsc));
                 }
             };
             constexpr int kStep = U * NTB;
             for (int rb = r0; rb < r1; rb += 2 * kStep) {
-                if (rb + kStep < r1) tb_load<NTB>(bb, rkey, rw, base, rb + kStep, r1, tid);
+                if (rb + kStep < r1) tb_load<NTB, U>(bb, V.rec, base, rb + kStep, r1, tid);
                 run(ba, rb);
                 if (rb + kStep >= r1) break;
-                if (rb + 2 * kStep < r1) tb_load<NTB>(ba, rkey, rw, base, rb + 2 * kStep, r1, tid);
+                if (rb + 2 * kStep < r1) tb_load<NTB, U>(ba, V.rec, base, rb + 2 * kStep, r1, tid);
                 run(bb, rb + kStep);
             }
         }
