@@ -56,7 +56,8 @@ typedef enum {
 
 typedef enum {
     MBIR_MODE_AUTO = 0,          /* TAB when the leg table fits, else OTF */
-    MBIR_MODE_OTF = 1,           /* travel times solved in registers on every apply */
+    MBIR_MODE_OTF = 1,           /* travel times solved on every apply (into a workspace of at most 64 MB where the
+                                  * distinct |x_c - u| fit one, pair by pair otherwise) */
     MBIR_MODE_TAB = 2            /* legs solved once per geometry, kept in device memory */
 } mbir_mode;
 

@@ -278,7 +278,12 @@ cudaError_t launch_backproject(const mbir_geometry* g, const float* e_pad, const
 {
     const bool bf = g->P.precision == MBIR_PREC_BF16;
     if (g->d_tb4_bop) return launch_backproject_tcs(g, e_pad, e_bf, b, st);
-    if (g->P.mode == MBIR_MODE_TAB)
+    bool legs = g->P.mode == MBIR_MODE_TAB;
+    if (!legs) {
+        const cudaError_t ce = solve_otf_legs(g, st, &legs);
+        if (ce != cudaSuccess) return ce;
+    }
+    if (legs)
         return bf ? launch_bwd_nl<kModeTAB, true>(g, e_bf, b, st) : launch_bwd_nl<kModeTAB, false>(g, e_pad, b, st);
     return bf ? launch_bwd_nl<kModeOTF, true>(g, e_bf, b, st) : launch_bwd_nl<kModeOTF, false>(g, e_pad, b, st);
 }
@@ -369,7 +374,10 @@ cudaError_t load_backproject_partials(const mbir_geometry* g)
     cudaFuncAttributes a;
     cudaError_t e = cudaFuncGetAttributes(&a, backproject_reduce_kernel);
     if (e != cudaSuccess) return e;
-    if (g->P.mode == MBIR_MODE_TAB) return cudaFuncGetAttributes(&a, backproject_kernel<1, kModeTAB, false>);
+    if (g->d_hvals) e = load_otf_legs(g);
+    if (e != cudaSuccess) return e;
+    if (g->P.mode == MBIR_MODE_TAB || g->d_hvals)
+        return cudaFuncGetAttributes(&a, backproject_kernel<1, kModeTAB, false>);
     if (g->P.L <= 2) return cudaFuncGetAttributes(&a, backproject_kernel<2, kModeOTF, false>);
     if (g->P.L <= 4) return cudaFuncGetAttributes(&a, backproject_kernel<4, kModeOTF, false>);
     return cudaFuncGetAttributes(&a, backproject_kernel<8, kModeOTF, false>);
@@ -379,7 +387,12 @@ cudaError_t launch_backproject_partials(const mbir_geometry* g, const float* e_p
                                         float* b, float* partial, cudaStream_t st)
 {
     const bool bf = g->P.precision == MBIR_PREC_BF16;
-    if (g->P.mode == MBIR_MODE_TAB)
+    bool legs = g->P.mode == MBIR_MODE_TAB;
+    if (!legs) {
+        const cudaError_t ce = solve_otf_legs(g, st, &legs);
+        if (ce != cudaSuccess) return ce;
+    }
+    if (legs)
         return bf ? launch_bwd_partials_t<1, kModeTAB, true>(g, e_bf, b, partial, st)
                   : launch_bwd_partials_t<1, kModeTAB, false>(g, e_pad, b, partial, st);
     if (g->P.L <= 2)

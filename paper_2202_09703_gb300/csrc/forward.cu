@@ -253,7 +253,12 @@ cudaError_t launch_forward(const mbir_geometry* g, const float* x, float* y_f32,
     if (g->d_tf4_bop) return launch_forward_tcs(g, x, y_f32, y_bf16, out_stride, st);
     if (g->d_rec_key) return launch_forward_sorted(g, x, y_f32, y_bf16, out_stride, st);
     const bool bf = g->P.precision == MBIR_PREC_BF16;
-    if (g->P.mode == MBIR_MODE_TAB)
+    bool legs = g->P.mode == MBIR_MODE_TAB;
+    if (!legs) {
+        const cudaError_t ce = solve_otf_legs(g, st, &legs);
+        if (ce != cudaSuccess) return ce;
+    }
+    if (legs)
         return bf ? launch_fwd_nl<kModeTAB, true>(g, x, y_f32, y_bf16, out_stride, st)
                   : launch_fwd_nl<kModeTAB, false>(g, x, y_f32, y_bf16, out_stride, st);
     return bf ? launch_fwd_nl<kModeOTF, true>(g, x, y_f32, y_bf16, out_stride, st)

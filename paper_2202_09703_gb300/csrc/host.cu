@@ -1,6 +1,6 @@
 // Host side of the library: argument validation, the pulse table (built once
 // in FP64 by FFT), per-row and per-transducer tables, device uploads, the
-// leg table of TAB mode, and the C ABI entry points that manage handles.
+// leg table of TAB mode (of OTF mode: its list of offsets and workspace), and the C ABI entry points that manage handles.
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -17,6 +17,7 @@ using mbir::RowInfo;
 namespace {
 
 constexpr double kPi = 3.14159265358979323846;
+constexpr size_t kOtfLegBytes = (size_t)64 << 20;   // largest leg workspace of the on-the-fly form
 
 float2 split_df(double v)
 {
@@ -169,7 +170,7 @@ void free_geometry(mbir_geometry* g)
 {
     if (!g) return;
     void* ptrs[] = {g->d_rows, g->d_colx, g->d_pos, g->d_txpos, g->d_rxpos, g->d_tab, g->d_tab_bf16,
-                    g->d_legs, g->d_hidx, g->d_direct, g->d_dinv, g->d_status, g->w_e, g->w_q,
+                    g->d_legs, g->d_hidx, g->d_hvals, g->d_hsign, g->d_direct, g->d_dinv, g->d_status, g->w_e, g->w_q,
                     g->w_b, g->w_grad, g->w_gprev, g->w_d, g->w_part, g->w_scal, g->w_ebf,
                     g->w_msq, g->w_d2, g->w_xalt, g->w_y, g->w_x, g->w_g, g->w_hist, g->d_items, g->w_bpart,
                     g->d_rec_off, g->d_rec_key, g->d_rec_w, g->d_tc_key, g->d_tc_w, g->d_runs, g->d_win_order, g->d_win_counter,
@@ -414,7 +415,8 @@ int mbir_create_geometry(const mbir_geometry_desc* d, void* stream, mbir_geometr
         size_t tab_bytes = (size_t)P.H * (u0.size() + u1.size()) * sizeof(float4);
         if (mode == MBIR_MODE_AUTO) mode = (tab_bytes <= ((size_t)4 << 30)) ? MBIR_MODE_TAB : MBIR_MODE_OTF;
         if (tilted && mode != MBIR_MODE_TAB) { free_geometry(g); return MBIR_ERR_UNSUPPORTED; }
-        if (mode == MBIR_MODE_TAB) {
+        // the on-the-fly form's applies solve into a workspace of at most half the L2, which keeps it there
+        if (mode == MBIR_MODE_TAB || tab_bytes <= kOtfLegBytes) {
             auto nearest = [tol](const std::vector<double>& u, double x) {
                 size_t i = std::lower_bound(u.begin(), u.end(), x - tol) - u.begin();
                 if (i + 1 < u.size() && std::fabs(u[i + 1] - x) < std::fabs(u[i] - x)) ++i;
@@ -454,6 +456,27 @@ int mbir_create_geometry(const mbir_geometry_desc* d, void* stream, mbir_geometr
     UP(g->d_dinv, dinv);
     std::vector<int> status(4, 0);
     UP(g->d_status, status);
+    if (mode == MBIR_MODE_OTF && !hvals.empty()) {
+        // without memory for the workspace the applies solve pair by pair
+        size_t wsb = sizeof(float4) * (size_t)P.H * P.nh;
+        ce = cudaMalloc((void**)&g->d_legs, wsb);
+        if (ce == cudaSuccess) ce = upload(&g->d_hidx, hidx.data(), hidx.size(), &wsb);
+        if (ce == cudaSuccess) ce = upload(&g->d_hsign, hsign.data(), hsign.size(), &wsb);
+        if (ce == cudaSuccess) ce = upload(&g->d_hvals, hvals.data(), hvals.size(), &wsb);
+        if (ce != cudaSuccess && ce != cudaErrorMemoryAllocation) { free_geometry(g); return cuda_err(ce); }
+        if (ce == cudaSuccess) {
+            bytes += wsb;
+        } else {
+            cudaGetLastError();
+            cudaFree(g->d_legs);
+            cudaFree(g->d_hidx);
+            cudaFree(g->d_hsign);
+            cudaFree(g->d_hvals);
+            g->d_legs = nullptr;
+            g->d_hidx = g->d_hsign = nullptr;
+            g->d_hvals = nullptr;
+        }
+    }
     if (mode == MBIR_MODE_TAB) {
         UP(g->d_hidx, hidx);
         float2* d_hv = nullptr;

@@ -351,8 +351,10 @@ struct mbir_geometry {
     int* d_rxpos;          // K position index per A-scan receiver
     float2* d_tab;         // Gt x (Q+1) x Tw4 pulse table, float2 = (plane g, plane g+1)
     __nv_bfloat162* d_tab_bf16;
-    float4* d_legs;        // TAB: H x nh legs
-    int* d_hidx;           // TAB: npos x W index into the |h| list
+    float4* d_legs;        // TAB: H x nh legs; OTF: workspace for them, solved again by every apply (d_hvals)
+    int* d_hidx;           // npos x W index into the |h| list
+    float2* d_hvals;       // OTF with a leg workspace: the |h| list, and its side flags (all 0)
+    int* d_hsign;
     float* d_direct;       // n_rx x Mp direct-arrival columns (eq. 1)
     float* d_dinv;         // n_rx: 1 / |d_j|^2 (0 if empty)
     int* d_status;         // device error flag (bounded waits)
@@ -459,6 +461,8 @@ struct mbir_geometry {
 namespace mbir {
 // launchers implemented in apply.cu
 cudaError_t launch_build_legs(const mbir_geometry* g, const int* d_hsign, const float2* d_hvals, cudaStream_t st);
+cudaError_t solve_otf_legs(const mbir_geometry* g, cudaStream_t st, bool* table);
+cudaError_t load_otf_legs(const mbir_geometry* g);
 cudaError_t launch_backproject(const mbir_geometry* g, const float* e_pad, const __nv_bfloat16* e_bf,
                                float* b, cudaStream_t st);
 cudaError_t launch_forward(const mbir_geometry* g, const float* x, float* y_f32, __nv_bfloat16* y_bf16,

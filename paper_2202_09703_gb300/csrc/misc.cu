@@ -38,6 +38,30 @@ cudaError_t launch_build_legs(const mbir_geometry* g, const int* d_hsign, const 
     return cudaGetLastError();
 }
 
+// On-the-fly form: every leg of this apply into the geometry's workspace, one per (row, distinct |x_c - u|),
+// on the apply's stream; *table is false when the geometry has no such workspace and its kernels solve the
+// legs pair by pair.
+//
+// Pair by pair an apply solves one leg per (pixel, A-scan) and more: 256x512 with 64 x 16 A-scans, 143 M in
+// A^T and 268 M in A x, about 1000 instructions each.  A scanner that moves in steps related to the pixel
+// pitch meets the same |x_c - u| over and over: 0.4 M legs there, which the applies then read from the L2.
+// Measured there: A x 28.7 -> 10.7 ms, A^T 7.13 -> 2.26 ms.  A table never holds more legs than the pairs ask
+// for; its limit (kOtfLegBytes, host.cu) is half the L2, beyond which its reads would go to memory.
+cudaError_t solve_otf_legs(const mbir_geometry* g, cudaStream_t st, bool* table)
+{
+    *table = g->P.mode == MBIR_MODE_OTF && g->d_hvals;
+    return *table ? launch_build_legs(g, g->d_hsign, g->d_hvals, st) : cudaSuccess;
+}
+
+// Loads the kernel that solve_otf_legs runs for g (see load_backproject_partials).
+cudaError_t load_otf_legs(const mbir_geometry* g)
+{
+    cudaFuncAttributes a;
+    if (g->P.L <= 2) return cudaFuncGetAttributes(&a, build_legs_kernel<2>);
+    if (g->P.L <= 4) return cudaFuncGetAttributes(&a, build_legs_kernel<4>);
+    return cudaFuncGetAttributes(&a, build_legs_kernel<8>);
+}
+
 template <int NL, int MODE>
 __global__ void pair_quantities_kernel(GeomParams P, DevPtrs D, const int* __restrict__ pix, const int* __restrict__ ks,
                                        int n, double* __restrict__ T, float* __restrict__ gam, float* __restrict__ w)
