@@ -212,21 +212,27 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int d = c + j;                              // column within the block
-                    const float u = __shfl_sync(full, (v[j] * i0) * it, (lane - d) & 31);
+                    const float u = __shfl_sync(full, v[j], (lane - d) & 31);
                     if (lane >= d) lo += u;
                     else hi += u;
                 }
             }
-            part[warp * kTsPart + lane] = lo;
-            part[warp * kTsPart + 32 + lane] = hi;
+            part[warp * kTsPart + lane] = (lo * i0) * it;
+            part[warp * kTsPart + 32 + lane] = (hi * i0) * it;
         }
         tc_fence_before();
         __syncthreads();
+        // (no barrier at the end: the caller's next one comes before part is written or sY is read)
         for (int o = tid; o < kTsTile + T.ntap - 1; o += blockDim.x) {
+            // the blocks that hold output o: per column block the lane quarter of its offset, as a row below 32,
+            // and the quarter before, as a row past 32
             float acc = 0.0f;
-            for (int w = 0; w < kTsEpiWarps; ++w) {
-                const int r = o - ((w & 3) * 32 + (w >> 2) * cq);
-                if (r >= 0 && r < 32 + cq - 1) acc += part[w * kTsPart + r];
+#pragma unroll
+            for (int b = 0; b < kTsEpiWarps / 4; ++b) {
+                const int r = o - b * cq, q1 = r >> 5, r1 = r & 31;
+                const float* pw = part + (b * 4 + q1) * kTsPart + r1;
+                if (q1 >= 1 && q1 <= 4 && r1 < cq - 1) acc += pw[32 - kTsPart];
+                if (q1 >= 0 && q1 <= 3) acc += pw[0];
             }
             sY[(tp * kTsTile + 1 + o) & (kTsYRing - 1)] += acc;
         }
@@ -287,9 +293,14 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
                 ww = WT{};
             }
         };
+        auto gather = [&](int s) {
+            xq[s] = kq[s].y != kTcNone ? ld_x<FV>(xg + (kq[s].x & kTcPixelMask)) : 0.0f;
+        };
         warp_range(0);
 #pragma unroll
         for (int s = 0; s < kTsRing; ++s) issue(kq[s], wq[s], s);
+#pragma unroll
+        for (int s = 0; s < kTsXAhead; ++s) gather(s);
 
         int pend = -1, pend_se = 0;                      // tile whose products wait in tensor memory
         for (int t = 0; t < ntile; ++t) {
@@ -318,17 +329,13 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
                 float* Sb = sS - (int)(tcr[t] & 0xffffu);
                 float bsum = 0.0f;
                 // x gathered kTsXAhead batches ahead of its use, the records kTsRing batches ahead
-#pragma unroll
-                for (int s = 0; s < kTsXAhead; ++s)
-                    xq[s] = kq[s].y != kTcNone ? ld_x<FV>(xg + (kq[s].x & kTcPixelMask)) : 0.0f;
                 for (int b0 = 0; b0 < nb; b0 += kTsRing) {
 #pragma unroll
                     for (int u = 0; u < kTsRing; ++u) {
                         const int b = b0 + u;
                         if (b >= nb) break;
                         if (b + kTsXAhead < nb) {
-                            const int sn = (u + kTsXAhead) % kTsRing;
-                            xq[sn] = kq[sn].y != kTcNone ? ld_x<FV>(xg + (kq[sn].x & kTcPixelMask)) : 0.0f;
+                            gather((u + kTsXAhead) % kTsRing);
                         }
                         const uint2 kk = kq[u];
                         const bool valid = kk.y != kTcNone;
@@ -422,16 +429,23 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
 #pragma unroll
                 for (int s = 0; s < kTsRing; ++s) issue(kq[s], wq[s], s);
             }
-            if (!live) continue;
+            if (!live) {
+#pragma unroll
+                for (int s = 0; s < kTsXAhead; ++s) gather(s);
+                continue;
+            }
             __syncthreads();                             // every record of the tile is in S
             // ---- the previous tile's products -> y (they ran during this tile's scatter); the samples before
             // this tile's first are then final
             if (pend >= 0) {
                 epilogue(pend, pend_se);
-                __syncthreads();
-                flush((pend + 1) * kTsTile + 1, pend * kTsTile + 1);
             }
-            if (*abort_flag) break;
+            // The first x of the next tile are gathered while this one is converted and multiplied, and its
+            // conversion starts without waiting for the previous tile's sums and stores: three barriers per tile
+            // instead of five.  256x512 FP32 0.574 -> 0.562 ms, 512x1024 FP32 8.96 -> 8.82 ms, BF16 8.21 -> 8.01 ms
+            // (with the block sums reduced to the blocks that hold an output).
+#pragma unroll
+            for (int s = 0; s < kTsXAhead; ++s) gather(s);
             // ---- S -> A operand in tensor memory, S cleared as read
             int se = 0;
             if (!BF16) {
@@ -471,6 +485,7 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
             }
             tc_fence_before();
             __syncthreads();
+            if (*abort_flag) break;
             if (tid == 32 * (kTsWarps - 1)) {
                 tc_fence_after();
                 // (one thread issues dozens of products: the descriptors are stepped, not rebuilt)
@@ -486,6 +501,9 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
                 }
                 umma_commit(smem_u32(smem));
             }
+            // the previous tile's samples before this tile's first are final; the next scatter's tau = t0 taps
+            // lie at most 382 + Tw samples past them, in other slots of the ring
+            if (pend >= 0) flush((pend + 1) * kTsTile + 1, pend * kTsTile + 1);
             pend = t;
             pend_se = se;
         }
