@@ -8,7 +8,9 @@
 // written by a conflict-free scatter (each bound is owned by exactly one row),
 // then each warp produces its spans with counted loops over those runs.
 // Every output sample is owned by one lane: no atomics, a fixed summation
-// order, bitwise reproducible results.
+// order, bitwise reproducible results.  Serves the geometries without stored
+// records that forward_legs.cu does not take (no leg table, or a tile that
+// reaches too many attenuation planes).
 #include <algorithm>
 
 #include "device_common.cuh"
@@ -258,6 +260,7 @@ cudaError_t launch_forward(const mbir_geometry* g, const float* x, float* y_f32,
         const cudaError_t ce = solve_otf_legs(g, st, &legs);
         if (ce != cudaSuccess) return ce;
     }
+    if (g->d_fl_tab) return launch_forward_legs(g, x, y_f32, y_bf16, out_stride, st);
     if (legs)
         return bf ? launch_fwd_nl<kModeTAB, true>(g, x, y_f32, y_bf16, out_stride, st)
                   : launch_fwd_nl<kModeTAB, false>(g, x, y_f32, y_bf16, out_stride, st);

@@ -1,0 +1,404 @@
+// A x without stored records, from a table of legs (the on-the-fly form's workspace, or TAB mode without
+// records).  Every tap of a pair shares one table phase, so with the pairs of an A-scan grouped by first tap n0
+//     S[n0][col] = sum of the pairs' bilinear corner weights on table column col times x,
+//     y[n0 + 1 + m] += sum_col S[n0][col] T[col][m],       col = plane * (Q + 1) + phase,
+// for one tile of 128 values of n0 after another.
+//
+// Pairs: in one layer the delay grows with depth, so each (column, layer) of the image holds a tile's pixels in
+// one run of rows; a thread keeps a cursor per (column, layer) and walks on from it, tile after tile, so each
+// pair is evaluated once, and none past the record's end.  Nothing is sorted, compacted or staged.
+//
+// S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
+// first one's old value), at a scale that the largest |x| and the number of pixels keep from overflow: exact, so
+// the result does not depend on the order of the additions and every output bit is reproducible.  The product
+// with the table is FP32 on the CUDA cores: it is a short convolution per column, which a thread does for four
+// outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
+// would not (3e-7 against 1.5e-7 from FP64).
+//
+// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), after the legs: 3.3 ms against 10.7 ms of
+// forward_kernel, which gathers every tap of every pair.  The product takes about half of it (its FP32 rate and
+// the shared-memory loads that feed it), the walk over the pairs the rest (latency of the legs and the atomics).
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "device_common.cuh"
+
+namespace mbir {
+
+constexpr int kFlTile = 128;                     // values of n0 per tile
+constexpr int kFlThreads = 1024;
+constexpr int kFlMaxTiles = 512;                 // tiles of an A-scan (set-up's shared memory)
+
+// Shared memory: S as low and high words (columns of 128), then the edge taps' words, the share sums, carries,
+// row flags and cursors.
+struct FlLayout {
+    int ng, ncg;             // groups of four outputs; shares of the columns
+    size_t off_hi, off_edge, off_part, off_carry, off_bad, off_cur, smem;
+};
+__host__ __device__ inline FlLayout fl_layout(const GeomParams& P, int kw)
+{
+    FlLayout L;
+    L.ng = (kFlTile + P.Tw - 1 + 3) / 4;
+    L.ncg = kFlThreads / L.ng;
+    L.off_hi = (size_t)kw * kFlTile * 4;
+    L.off_edge = 2 * L.off_hi;
+    L.off_part = L.off_edge + 2 * kFlTile * 4;
+    L.off_carry = L.off_part + (size_t)L.ncg * L.ng * 16;
+    L.off_bad = L.off_carry + 2 * kFlTile * 4;
+    L.off_cur = L.off_bad + (kFlTile + 4) * 4;
+    L.smem = L.off_cur + (((size_t)P.W * P.n_seg * 2 + 15) & ~(size_t)15);
+    return L;
+}
+
+// *out = bits of the largest finite |x| (zero before)
+__global__ void fl_xmax_kernel(int N, const float* __restrict__ x, unsigned int* __restrict__ out)
+{
+    unsigned int m = 0;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
+        const unsigned int b = __float_as_uint(x[i]) & 0x7fffffffu;
+        if (b < 0x7f800000u) m = max(m, b);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m) atomicMax(out, m);
+}
+
+// v 2^e (e split in two: 2^e itself may be out of range)
+__device__ __forceinline__ float fl_scale(float v, int e)
+{
+    const int e1 = e >> 1;
+    return v * __int_as_float((e1 + 127) << 23) * __int_as_float((e - e1 + 127) << 23);
+}
+
+// The word at `at` and its high word (`hi` words further) += q
+__device__ __forceinline__ void fl_add(unsigned int* at, size_t hi, long long q)
+{
+    const unsigned int l = (unsigned int)q;
+    unsigned int h = (unsigned int)(q >> 32);
+    const unsigned int old = atomicAdd(at, l);
+    h += old + l < old ? 1u : 0u;
+    if (h) atomicAdd(at + hi, h);
+}
+
+__device__ __forceinline__ long long fl_word(unsigned int lo, unsigned int hi)
+{
+    return (long long)((unsigned long long)hi << 32 | lo);
+}
+
+__device__ __forceinline__ Leg fl_leg(float4 v) { return Leg{v.x, v.y, v.z, v.w}; }
+
+// Block (A-scan, chunk of tiles): tiles [ta, tb), and the one before for the taps that reach past it.
+__global__ void __launch_bounds__(kFlThreads, 1)
+    forward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint32_t* __restrict__ crange,
+                        const float* __restrict__ x, const unsigned int* __restrict__ xmax, int sbits, int ebits,
+                        int kwmax, int per, float* __restrict__ y_f32, __nv_bfloat16* __restrict__ y_bf16,
+                        int out_stride)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const FlLayout L = fl_layout(P, kwmax);
+    unsigned int* lo = reinterpret_cast<unsigned int*>(smem);
+    unsigned int* edge = reinterpret_cast<unsigned int*>(smem + L.off_edge);
+    float* part = reinterpret_cast<float*>(smem + L.off_part);
+    float* carry = reinterpret_cast<float*>(smem + L.off_carry);
+    int* bad = reinterpret_cast<int*>(smem + L.off_bad);                 // rows with a non-finite x; [128]: any
+    unsigned short* cur = reinterpret_cast<unsigned short*>(smem + L.off_cur);
+    const size_t hiw = L.off_hi / 4;
+    const int tid = threadIdx.x, k = blockIdx.x;
+    const int ntile = (P.M + kFlTile - 1) / kFlTile;
+    const int ta = blockIdx.y * per, tb = min(ta + per, ntile), t0 = max(ta - 1, 0);
+    const int R = P.Q + 1, dR = P.G > 1 ? R : 0, ncur = P.W * P.n_seg;
+    const int* htx = D.hidx + (size_t)__ldg(D.txpos + k / P.n_rx) * P.W;
+    const int* hrx = D.hidx + (size_t)__ldg(D.rxpos + k) * P.W;
+    // fixed-point scale: |x| < 2^ex and weights of at most 1 (2 with rounding), W x H of them, stay below 2^62
+    int ex = 0;
+    frexpf(__uint_as_float(__ldg(xmax)), &ex);
+    const int se = sbits - ex;
+
+    auto store = [&](int n, float v) {
+        if (y_f32) y_f32[(size_t)k * out_stride + n] = v;
+        else y_bf16[(size_t)k * out_stride + n] = __float2bfloat16_rn(v);
+    };
+    for (size_t i = tid; i < L.off_part / 4; i += kFlThreads) lo[i] = 0u;
+    if (tid < 2 * kFlTile) carry[tid] = 0.0f;
+    if (tid <= kFlTile) bad[tid] = 0;
+    if (ta == 0 && tid == 0) store(0, 0.0f);
+    if (tb == ntile)
+        for (int n = P.M + tid; n < out_stride; n += kFlThreads) store(n, 0.0f);
+    // cursors: the first row of each (layer, column) whose pair starts in tile t0 or later
+    for (int j = tid; j < ncur; j += kFlThreads) {
+        const int sg = j / P.W, col = j - sg * P.W;
+        int a = P.seg_row[sg], b = P.seg_row[sg + 1];
+        if (t0 == 0) b = a;
+        const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
+        while (a < b) {
+            const int mid = (a + b) >> 1;
+            const float4* lr = D.legs + (size_t)mid * P.nh;
+            if (make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)), 1.0f).n0 < t0 * kFlTile) a = mid + 1;
+            else b = mid;
+        }
+        cur[j] = (unsigned short)a;
+    }
+    __syncthreads();
+
+    const int cg = tid / L.ng, og = tid - cg * L.ng;
+    int par = 0;
+    for (int t = t0; t < tb; ++t) {
+        const int ts = t * kFlTile;
+        const uint32_t cr = __ldg(crange + (size_t)k * ntile + t);
+        const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
+        if (kw > 0) {
+            // ---- the tile's pairs into S
+            for (int j = tid; j < ncur; j += kFlThreads) {
+                const int sg = j / P.W, col = j - sg * P.W, end = P.seg_row[sg + 1];
+                int row = cur[j];
+                if (row >= end) continue;
+                const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
+                const float4* lr = D.legs + (size_t)row * P.nh;
+                float4 a = __ldg(lr + ht), b = __ldg(lr + hr);
+                float xv = __ldg(x + (size_t)row * P.W + col);
+                for (;;) {
+                    // the next row's legs load while this one's pair is evaluated
+                    lr += P.nh;
+                    float4 an = a, bn = b;
+                    float xn = 0.0f;
+                    if (row + 1 < end) {
+                        an = __ldg(lr + ht);
+                        bn = __ldg(lr + hr);
+                        xn = __ldg(x + (size_t)(row + 1) * P.W + col);
+                    }
+                    const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
+                    const int n0r = pr.n0 - ts;
+                    if (n0r >= kFlTile) break;
+                    const float wx = pr.w * xv;
+                    if (wx != 0.0f && n0r >= 0 && pr.n0 + 1 < P.M && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) {
+                        if (fabsf(wx) <= 3.4028235e38f) {
+                            const float p1 = pr.psi, p0 = 1.0f - pr.psi;
+                            unsigned int* s = lo + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
+                            const float wa = wx * pr.w0, wb = wx * pr.w1;
+                            fl_add(s, hiw, __float2ll_rn(fl_scale(wa * p0, se)));
+                            fl_add(s + kFlTile, hiw, __float2ll_rn(fl_scale(wb * p0, se)));
+                            if (dR) {
+                                fl_add(s + dR * kFlTile, hiw, __float2ll_rn(fl_scale(wa * p1, se)));
+                                fl_add(s + (dR + 1) * kFlTile, hiw, __float2ll_rn(fl_scale(wb * p1, se)));
+                            }
+                            if (pr.flag0) {
+                                // tau = t0 exactly: the last tap of the upper phase lies outside the window
+                                const float* tl = ftab + (size_t)(pr.gi * R + pr.r + 1) * P.Tw4 + P.Tw - 1;
+                                const float ev = wb * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4));
+                                fl_add(edge + n0r, kFlTile, __float2ll_rn(fl_scale(ev, se - ebits)));
+                            }
+                        } else {
+                            bad[n0r] = 1;
+                            bad[kFlTile] = 1;
+                        }
+                    }
+                    if (pr.n0 + 1 >= P.M) row = end - 1;             // the rows below start later still
+                    if (++row >= end) break;
+                    a = an;
+                    b = bn;
+                    xv = xn;
+                }
+                cur[j] = (unsigned short)row;
+            }
+            __syncthreads();
+            // ---- S as FP32 in place of its low words
+            uint4* l4 = reinterpret_cast<uint4*>(lo);
+            uint4* h4 = reinterpret_cast<uint4*>(lo + hiw);
+            for (int i = tid; i < kw * (kFlTile / 4); i += kFlThreads) {
+                const uint4 l = l4[i], h = h4[i];
+                h4[i] = make_uint4(0u, 0u, 0u, 0u);
+                l4[i] = make_uint4(__float_as_uint(fl_scale(__ll2float_rn(fl_word(l.x, h.x)), -se)),
+                                   __float_as_uint(fl_scale(__ll2float_rn(fl_word(l.y, h.y)), -se)),
+                                   __float_as_uint(fl_scale(__ll2float_rn(fl_word(l.z, h.z)), -se)),
+                                   __float_as_uint(fl_scale(__ll2float_rn(fl_word(l.w, h.w)), -se)));
+            }
+            __syncthreads();
+            // ---- outputs 4 og .. 4 og + 3 of this thread's columns: sum_m S[o - m] T[m], four taps at a time
+            // against the blocks of four values of S at and below the output
+            if (cg < L.ncg) {
+                float y0 = 0.f, y1 = 0.f, y2 = 0.f, y3 = 0.f;
+                const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+                const int ntb = P.Tw4 / 4;
+                for (int c = cg; c < kw; c += L.ncg) {
+                    const float4* S = reinterpret_cast<const float4*>(lo + (size_t)c * kFlTile);
+                    const float4* T = reinterpret_cast<const float4*>(ftab + (size_t)(c_lo + c) * P.Tw4);
+                    float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+                    float4 h = og < kFlTile / 4 ? S[og] : zero;
+#pragma unroll 4
+                    for (int mb = 0; mb < ntb; ++mb) {
+                        const int l = og - mb - 1;
+                        const float4 b = (unsigned)l < (unsigned)(kFlTile / 4) ? S[l] : zero;
+                        const float4 w = __ldg(T + mb);
+                        a0 = fmaf(h.x, w.x, fmaf(b.w, w.y, fmaf(b.z, w.z, fmaf(b.y, w.w, a0))));
+                        a1 = fmaf(h.y, w.x, fmaf(h.x, w.y, fmaf(b.w, w.z, fmaf(b.z, w.w, a1))));
+                        a2 = fmaf(h.z, w.x, fmaf(h.y, w.y, fmaf(h.x, w.z, fmaf(b.w, w.w, a2))));
+                        a3 = fmaf(h.w, w.x, fmaf(h.z, w.y, fmaf(h.y, w.z, fmaf(h.x, w.w, a3))));
+                        h = b;
+                    }
+                    y0 += a0;
+                    y1 += a1;
+                    y2 += a2;
+                    y3 += a3;
+                }
+                reinterpret_cast<float4*>(part)[cg * L.ng + og] = make_float4(y0, y1, y2, y3);
+            }
+            __syncthreads();
+        }
+        // ---- the shares' sums, the previous tile's carry and the edge taps -> y; taps past this tile carry on
+        if (tid < 2 * kFlTile) {
+            float v = 0.0f;
+            if (kw > 0 && tid < 4 * L.ng) {
+                for (int c = 0; c < L.ncg; ++c) v += part[c * L.ng * 4 + tid];
+                const int r = tid - (P.Tw - 1);
+                if (r >= 0 && r < kFlTile)
+                    v -= fl_scale(__ll2float_rn(fl_word(edge[r], edge[kFlTile + r])), ebits - se);
+                if (bad[kFlTile])
+                    for (int q = max(r, 0); q <= min(tid, kFlTile - 1); ++q)
+                        if (bad[q]) v = __uint_as_float(0x7fc00000u);
+            }
+            if (tid < kFlTile) {
+                const int n = ts + 1 + tid;
+                v += carry[par * kFlTile + tid];
+                if (t >= ta && n < P.M) store(n, v);
+            } else {
+                carry[(par ^ 1) * kFlTile + tid - kFlTile] = v;
+            }
+        }
+        par ^= 1;
+        if (kw > 0) {
+            uint4* l4 = reinterpret_cast<uint4*>(lo);
+            for (int i = tid; i < kw * (kFlTile / 4); i += kFlThreads) l4[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
+        __syncthreads();
+        if (kw > 0) {
+            if (tid < 2 * kFlTile) edge[tid] = 0u;
+            if (tid <= kFlTile) bad[tid] = 0;
+            __syncthreads();
+        }
+    }
+}
+
+// Attenuation planes that the pairs of each (A-scan, tile) reach, as the range of table columns first | end << 16
+// (0: no pair); *wmax: the widest.  Block per A-scan.
+__global__ void fl_range_kernel(GeomParams P, DevPtrs D, uint32_t* __restrict__ crange, int* __restrict__ wmax)
+{
+    __shared__ int lo[kFlMaxTiles], hi[kFlMaxTiles];
+    const int k = blockIdx.x, ntile = (P.M + kFlTile - 1) / kFlTile;
+    for (int t = threadIdx.x; t < ntile; t += blockDim.x) {
+        lo[t] = 1 << 30;
+        hi[t] = -1;
+    }
+    __syncthreads();
+    const int tp = __ldg(D.txpos + k / P.n_rx), rp = __ldg(D.rxpos + k);
+    for (int v = threadIdx.x; v < P.W * P.H; v += blockDim.x) {
+        const int row = v / P.W, col = v - row * P.W;
+        const RowInfo ri = load_row(D.rows, row);
+        if (!(ri.tvert < (float)(P.M - 1))) continue;
+        const Pair pr = make_pair(P, get_leg<1, kModeTAB>(P, D, ri, row, col, tp),
+                                  get_leg<1, kModeTAB>(P, D, ri, row, col, rp), ri.tau);
+        if (pr.w == 0.0f || pr.n0 < 0 || pr.n0 + 1 >= P.M) continue;
+        const int t = pr.n0 / kFlTile;
+        if (pr.gi < lo[t]) atomicMin(lo + t, pr.gi);
+        if (pr.gi > hi[t]) atomicMax(hi + t, pr.gi);
+    }
+    __syncthreads();
+    const int R = P.Q + 1;
+    for (int t = threadIdx.x; t < ntile; t += blockDim.x) {
+        uint32_t r = 0;
+        if (hi[t] >= 0) {
+            const int a = lo[t] * R, b = (min(hi[t] + 1, P.G - 1) + 1) * R;
+            r = (uint32_t)a | (uint32_t)b << 16;
+            atomicMax(wmax, b - a);
+        }
+        crange[(size_t)k * ntile + t] = r;
+    }
+}
+
+// Set-up for a geometry without stored records: the column ranges (from the legs, solved here for the on-the-fly
+// form), the table by columns and the exponents.  cudaErrorNotSupported keeps forward_kernel.
+cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
+{
+    const GeomParams& P = g->P;
+    const int ntile = (P.M + kFlTile - 1) / kFlTile, R = P.Q + 1;
+    if (!g->d_legs || g->d_rec_key || g->d_tf4_bop || P.Tw > kFlTile || ntile > kFlMaxTiles || P.G * R > 65535 ||
+        P.H > 65535 || (long long)P.W * P.n_seg > 8192)
+        return cudaErrorNotSupported;
+    uint32_t* d_cr = nullptr;
+    float* d_tab = nullptr;
+    unsigned int* d_max = nullptr;
+    int wmax = 0;
+    const size_t ncr = (size_t)P.K * ntile, ntab = (size_t)P.G * R * P.Tw4;
+    cudaError_t e = cudaMalloc((void**)&d_cr, sizeof(uint32_t) * ncr);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_tab, sizeof(float) * ntab);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_max, sizeof(unsigned int));
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, sizeof(unsigned int), st);
+    if (e == cudaSuccess) {
+        bool table = false;
+        e = solve_otf_legs(g, st, &table);
+    }
+    if (e == cudaSuccess) {
+        fl_range_kernel<<<P.K, 1024, 0, st>>>(P, dev_ptrs(g), d_cr, reinterpret_cast<int*>(d_max));
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&wmax, d_max, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    float tmax = 0.0f;
+    if (e == cudaSuccess) {
+        const bool bf = P.precision == MBIR_PREC_BF16;
+        const int nq = P.Q * P.Tw + 1;
+        std::vector<float> tab(ntab, 0.0f);
+        for (int gp = 0; gp < P.G; ++gp)
+            for (int r = 0; r < R; ++r)
+                for (int m = 0; m < P.Tw; ++m) {
+                    float v = (float)g->tab_host[(size_t)gp * nq + m * P.Q + r];
+                    if (bf) v = __bfloat162float(__float2bfloat16_rn(v));
+                    tab[((size_t)gp * R + r) * P.Tw4 + m] = v;
+                    tmax = std::max(tmax, std::fabs(v));
+                }
+        e = cudaMemcpy(d_tab, tab.data(), sizeof(float) * ntab, cudaMemcpyHostToDevice);
+    }
+    const int kw = std::max(wmax, 1);
+    const size_t sm = fl_layout(P, kw).smem;
+    if (e == cudaSuccess && sm > 226 * 1024) e = cudaErrorNotSupported;     // a tile reaches too many planes
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(forward_legs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    if (e != cudaSuccess) {
+        cudaFree(d_cr);
+        cudaFree(d_tab);
+        cudaFree(d_max);
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
+    }
+    int np = 0, ext = 0;
+    while ((1LL << np) < (long long)P.W * P.H) ++np;
+    std::frexp(tmax, &ext);
+    g->fl_bits = 61 - np;
+    g->fl_ebits = std::max(ext, 0);
+    g->fl_kw = kw;
+    g->d_fl_crange = d_cr;
+    g->d_fl_tab = d_tab;
+    g->d_fl_max = d_max;
+    g->bytes += sizeof(uint32_t) * ncr + sizeof(float) * ntab + sizeof(unsigned int);
+    return cudaSuccess;
+}
+
+// One block per A-scan runs alone on its SM, so few A-scans leave SMs idle: their tiles are then cut into chunks
+// until there are four blocks per SM, of at least four tiles (each chunk repeats the tile before it).
+cudaError_t launch_forward_legs(const mbir_geometry* g, const float* x, float* yf, __nv_bfloat16* yb, int stride,
+                                cudaStream_t st)
+{
+    const GeomParams& P = g->P;
+    const int N = P.W * P.H, ntile = (P.M + kFlTile - 1) / kFlTile;
+    cudaError_t e = cudaMemsetAsync(g->d_fl_max, 0, sizeof(unsigned int), st);
+    if (e != cudaSuccess) return e;
+    fl_xmax_kernel<<<std::max(1, std::min((N + 1023) / 1024, g->n_sm)), 256, 0, st>>>(N, x, g->d_fl_max);
+    const int want = (4 * g->n_sm + P.K - 1) / P.K;
+    const int per = std::max((ntile + want - 1) / want, std::min(4, ntile));
+    forward_legs_kernel<<<dim3(P.K, (ntile + per - 1) / per), kFlThreads, fl_layout(P, g->fl_kw).smem, st>>>(
+        P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, x, g->d_fl_max, g->fl_bits, g->fl_ebits, g->fl_kw, per, yf, yb,
+        stride);
+    return cudaGetLastError();
+}
+
+}  // namespace mbir

@@ -392,6 +392,12 @@ struct mbir_geometry {
     int* d_bwd_counter;    // work counter of the A^T r launch
     float* h_bwd_cost;     // host copy: estimated A^T r cost per (16-row tile, 32-column tile, Tx position)
     int bwd_ntc;           // 32-column tiles per row of tiles
+    // A x without stored records, from the legs (forward_legs.cu): column ranges per (A-scan, tile), the table by
+    // columns, the largest |x| of the call; bits of the fixed-point sums and of the table, widest column range
+    uint32_t* d_fl_crange;
+    float* d_fl_tab;
+    unsigned int* d_fl_max;
+    int fl_bits, fl_ebits, fl_kw;
     // TAB-mode A x records sorted by first tap sample (see forward_tab.cu); with the tensor-core applies the
     // sorted records are replaced by their packed form (tc_apply.cuh), on the same per-A-scan offsets
     long long* d_rec_off;
@@ -463,6 +469,9 @@ namespace mbir {
 cudaError_t launch_build_legs(const mbir_geometry* g, const int* d_hsign, const float2* d_hvals, cudaStream_t st);
 cudaError_t solve_otf_legs(const mbir_geometry* g, cudaStream_t st, bool* table);
 cudaError_t load_otf_legs(const mbir_geometry* g);
+cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st);
+cudaError_t launch_forward_legs(const mbir_geometry* g, const float* x, float* yf, __nv_bfloat16* yb, int stride,
+                                cudaStream_t st);
 cudaError_t launch_backproject(const mbir_geometry* g, const float* e_pad, const __nv_bfloat16* e_bf,
                                float* b, cudaStream_t st);
 cudaError_t launch_forward(const mbir_geometry* g, const float* x, float* y_f32, __nv_bfloat16* y_bf16,
