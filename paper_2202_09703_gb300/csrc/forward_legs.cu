@@ -5,8 +5,10 @@
 // for one tile of 128 values of n0 after another.
 //
 // Pairs: in one layer the delay grows with depth, so each (column, layer) of the image holds a tile's pixels in
-// one run of rows; a thread keeps a cursor per (column, layer) and walks on from it, tile after tile, so each
-// pair is evaluated once, and none past the record's end.  Nothing is sorted, compacted or staged.
+// one run of rows; a cursor per (column, layer) moves on from tile to tile, so each pair is evaluated about
+// once, and none past the record's end.  A tile reaches only one or two layers of a column, so several warps take
+// every nsub-th row of a run each (one thread per run left most threads waiting at the barrier for runs of up to
+// 40 rows: 3.32 ms instead of 2.57).  Nothing is sorted, compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
 // first one's old value), at a scale that the largest |x| and the number of pixels keep from overflow: exact, so
@@ -15,8 +17,8 @@
 // outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
 // would not (3e-7 against 1.5e-7 from FP64).
 //
-// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), after the legs: 3.3 ms against 10.7 ms of
-// forward_kernel, which gathers every tap of every pair.  The product takes about half of it (its FP32 rate and
+// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.57 ms against 10.7 ms of
+// forward_kernel, which gathers every tap of every pair.  The product takes 0.95 ms of it (its FP32 rate and
 // the shared-memory loads that feed it), the walk over the pairs the rest (latency of the legs and the atomics).
 #include <algorithm>
 #include <cmath>
@@ -47,7 +49,7 @@ __host__ __device__ inline FlLayout fl_layout(const GeomParams& P, int kw)
     L.off_carry = L.off_part + (size_t)L.ncg * L.ng * 16;
     L.off_bad = L.off_carry + 2 * kFlTile * 4;
     L.off_cur = L.off_bad + (kFlTile + 4) * 4;
-    L.smem = L.off_cur + (((size_t)P.W * P.n_seg * 2 + 15) & ~(size_t)15);
+    L.smem = L.off_cur + (((size_t)P.W * P.n_seg * 8 + 15) & ~(size_t)15);
     return L;
 }
 
@@ -102,7 +104,9 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     float* part = reinterpret_cast<float*>(smem + L.off_part);
     float* carry = reinterpret_cast<float*>(smem + L.off_carry);
     int* bad = reinterpret_cast<int*>(smem + L.off_bad);                 // rows with a non-finite x; [128]: any
-    unsigned short* cur = reinterpret_cast<unsigned short*>(smem + L.off_cur);
+    // cursors of this tile and of the next, per (layer, column): row << 16 | its tile (0: not looked at)
+    unsigned int* cur = reinterpret_cast<unsigned int*>(smem + L.off_cur);
+    unsigned int* nxt = cur + (size_t)P.W * P.n_seg;
     const size_t hiw = L.off_hi / 4;
     const int tid = threadIdx.x, k = blockIdx.x;
     const int ntile = (P.M + kFlTile - 1) / kFlTile;
@@ -137,10 +141,13 @@ __global__ void __launch_bounds__(kFlThreads, 1)
             if (make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)), 1.0f).n0 < t0 * kFlTile) a = mid + 1;
             else b = mid;
         }
-        cur[j] = (unsigned short)a;
+        cur[j] = (unsigned int)a << 16;
+        nxt[j] = (unsigned int)P.seg_row[sg + 1] << 16;
     }
     __syncthreads();
 
+    // warps that share the rows of 32 columns: enough for every warp to take part
+    const int ngrp = (P.W + 31) / 32, nsub = min(16, max(1, kFlThreads / 32 / ngrp)), units = ngrp * nsub;
     const int cg = tid / L.ng, og = tid - cg * L.ng;
     int par = 0;
     for (int t = t0; t < tb; ++t) {
@@ -148,58 +155,70 @@ __global__ void __launch_bounds__(kFlThreads, 1)
         const uint32_t cr = __ldg(crange + (size_t)k * ntile + t);
         const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
         if (kw > 0) {
-            // ---- the tile's pairs into S
-            for (int j = tid; j < ncur; j += kFlThreads) {
-                const int sg = j / P.W, col = j - sg * P.W, end = P.seg_row[sg + 1];
-                int row = cur[j];
-                if (row >= end) continue;
+            // ---- the tile's pairs into S: a warp takes 32 columns and every sub-th row of each layer's run
+            for (int u = tid >> 5; u < units; u += kFlThreads / 32) {
+                const int sub = u / ngrp, col = (u - sub * ngrp) * 32 + (tid & 31);
+                if (col >= P.W) continue;
                 const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
-                const float4* lr = D.legs + (size_t)row * P.nh;
-                float4 a = __ldg(lr + ht), b = __ldg(lr + hr);
-                float xv = __ldg(x + (size_t)row * P.W + col);
-                for (;;) {
-                    // the next row's legs load while this one's pair is evaluated
-                    lr += P.nh;
-                    float4 an = a, bn = b;
-                    float xn = 0.0f;
-                    if (row + 1 < end) {
-                        an = __ldg(lr + ht);
-                        bn = __ldg(lr + hr);
-                        xn = __ldg(x + (size_t)(row + 1) * P.W + col);
+                for (int sg = 0; sg < P.n_seg; ++sg) {
+                    const int j = sg * P.W + col, end = P.seg_row[sg + 1];
+                    const unsigned int at = cur[j];
+                    if ((int)(at & 0xffffu) > t) {                         // the run starts in a later tile
+                        if (sub == 0) atomicMin(nxt + j, at);
+                        continue;
                     }
-                    const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
-                    const int n0r = pr.n0 - ts;
-                    if (n0r >= kFlTile) break;
-                    const float wx = pr.w * xv;
-                    if (wx != 0.0f && n0r >= 0 && pr.n0 + 1 < P.M && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) {
-                        if (fabsf(wx) <= 3.4028235e38f) {
-                            const float p1 = pr.psi, p0 = 1.0f - pr.psi;
-                            unsigned int* s = lo + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
-                            const float wa = wx * pr.w0, wb = wx * pr.w1;
-                            fl_add(s, hiw, __float2ll_rn(fl_scale(wa * p0, se)));
-                            fl_add(s + kFlTile, hiw, __float2ll_rn(fl_scale(wb * p0, se)));
-                            if (dR) {
-                                fl_add(s + dR * kFlTile, hiw, __float2ll_rn(fl_scale(wa * p1, se)));
-                                fl_add(s + (dR + 1) * kFlTile, hiw, __float2ll_rn(fl_scale(wb * p1, se)));
-                            }
-                            if (pr.flag0) {
-                                // tau = t0 exactly: the last tap of the upper phase lies outside the window
-                                const float* tl = ftab + (size_t)(pr.gi * R + pr.r + 1) * P.Tw4 + P.Tw - 1;
-                                const float ev = wb * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4));
-                                fl_add(edge + n0r, kFlTile, __float2ll_rn(fl_scale(ev, se - ebits)));
-                            }
-                        } else {
-                            bad[n0r] = 1;
-                            bad[kFlTile] = 1;
+                    int row = (int)(at >> 16) + sub;
+                    if (row >= end) continue;
+                    const float4* lr = D.legs + (size_t)row * P.nh;
+                    float4 a = __ldg(lr + ht), b = __ldg(lr + hr);
+                    float xv = __ldg(x + (size_t)row * P.W + col);
+                    for (;;) {
+                        // the next row's legs load while this one's pair is evaluated
+                        lr += (size_t)nsub * P.nh;
+                        float4 an = a, bn = b;
+                        float xn = 0.0f;
+                        if (row + nsub < end) {
+                            an = __ldg(lr + ht);
+                            bn = __ldg(lr + hr);
+                            xn = __ldg(x + (size_t)(row + nsub) * P.W + col);
                         }
+                        const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
+                        const int n0r = pr.n0 - ts;
+                        if (pr.n0 + 1 >= P.M) break;                       // the rows below start later still
+                        if (n0r >= kFlTile) {
+                            atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)(pr.n0 / kFlTile));
+                            break;
+                        }
+                        const float wx = pr.w * xv;
+                        if (wx != 0.0f && n0r >= 0 && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) {
+                            if (fabsf(wx) <= 3.4028235e38f) {
+                                const float p1 = pr.psi, p0 = 1.0f - pr.psi;
+                                unsigned int* s = lo + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
+                                const float wa = wx * pr.w0, wb = wx * pr.w1;
+                                fl_add(s, hiw, __float2ll_rn(fl_scale(wa * p0, se)));
+                                fl_add(s + kFlTile, hiw, __float2ll_rn(fl_scale(wb * p0, se)));
+                                if (dR) {
+                                    fl_add(s + dR * kFlTile, hiw, __float2ll_rn(fl_scale(wa * p1, se)));
+                                    fl_add(s + (dR + 1) * kFlTile, hiw, __float2ll_rn(fl_scale(wb * p1, se)));
+                                }
+                                if (pr.flag0) {
+                                    // tau = t0 exactly: the last tap of the upper phase lies outside the window
+                                    const float* tl = ftab + (size_t)(pr.gi * R + pr.r + 1) * P.Tw4 + P.Tw - 1;
+                                    const float ev = wb * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4));
+                                    fl_add(edge + n0r, kFlTile, __float2ll_rn(fl_scale(ev, se - ebits)));
+                                }
+                            } else {
+                                bad[n0r] = 1;
+                                bad[kFlTile] = 1;
+                            }
+                        }
+                        row += nsub;
+                        if (row >= end) break;
+                        a = an;
+                        b = bn;
+                        xv = xn;
                     }
-                    if (pr.n0 + 1 >= P.M) row = end - 1;             // the rows below start later still
-                    if (++row >= end) break;
-                    a = an;
-                    b = bn;
-                    xv = xn;
                 }
-                cur[j] = (unsigned short)row;
             }
             __syncthreads();
             // ---- S as FP32 in place of its low words
@@ -269,6 +288,10 @@ __global__ void __launch_bounds__(kFlThreads, 1)
         if (kw > 0) {
             uint4* l4 = reinterpret_cast<uint4*>(lo);
             for (int i = tid; i < kw * (kFlTile / 4); i += kFlThreads) l4[i] = make_uint4(0u, 0u, 0u, 0u);
+            for (int j = tid; j < ncur; j += kFlThreads) cur[j] = (unsigned int)P.seg_row[j / P.W + 1] << 16;
+            unsigned int* const was = cur;
+            cur = nxt;
+            nxt = was;
         }
         __syncthreads();
         if (kw > 0) {
