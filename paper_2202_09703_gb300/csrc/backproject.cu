@@ -283,6 +283,7 @@ cudaError_t launch_backproject(const mbir_geometry* g, const float* e_pad, const
         const cudaError_t ce = solve_otf_legs(g, st, &legs);
         if (ce != cudaSuccess) return ce;
     }
+    if (g->w_fl_acc) return launch_backproject_legs(g, e_pad, e_bf, b, st);
     if (legs)
         return bf ? launch_bwd_nl<kModeTAB, true>(g, e_bf, b, st) : launch_bwd_nl<kModeTAB, false>(g, e_pad, b, st);
     return bf ? launch_bwd_nl<kModeOTF, true>(g, e_bf, b, st) : launch_bwd_nl<kModeOTF, false>(g, e_pad, b, st);

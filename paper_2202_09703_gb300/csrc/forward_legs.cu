@@ -1,4 +1,4 @@
-// A x without stored records, from a table of legs (the on-the-fly form's workspace, or TAB mode without
+// A x and A^T r without stored records, from a table of legs (the on-the-fly form's workspace, or TAB mode without
 // records).  Every tap of a pair shares one table phase, so with the pairs of an A-scan grouped by first tap n0
 //     S[n0][col] = sum of the pairs' bilinear corner weights on table column col times x,
 //     y[n0 + 1 + m] += sum_col S[n0][col] T[col][m],       col = plane * (Q + 1) + phase,
@@ -8,7 +8,7 @@
 // one run of rows; a cursor per (column, layer) moves on from tile to tile, so each pair is evaluated about
 // once, and none past the record's end.  A tile reaches only one or two layers of a column, so several warps take
 // every nsub-th row of a run each (one thread per run left most threads waiting at the barrier for runs of up to
-// 40 rows: 3.32 ms instead of 2.57).  Nothing is sorted, compacted or staged.
+// 40 rows: 3.3 ms instead of 2.6).  Nothing is sorted, compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
 // first one's old value), at a scale that the largest |x| and the number of pixels keep from overflow: exact, so
@@ -17,7 +17,7 @@
 // outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
 // would not (3e-7 against 1.5e-7 from FP64).
 //
-// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.57 ms against 10.7 ms of
+// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.6 ms against 10.7 ms of
 // forward_kernel, which gathers every tap of every pair.  The product takes 0.95 ms of it (its FP32 rate and
 // the shared-memory loads that feed it), the walk over the pairs the rest (latency of the legs and the atomics).
 #include <algorithm>
@@ -53,12 +53,16 @@ __host__ __device__ inline FlLayout fl_layout(const GeomParams& P, int kw)
     return L;
 }
 
+__device__ __forceinline__ float fl_float(float v) { return v; }
+__device__ __forceinline__ float fl_float(__nv_bfloat16 v) { return __bfloat162float(v); }
+
 // *out = bits of the largest finite |x| (zero before)
-__global__ void fl_xmax_kernel(int N, const float* __restrict__ x, unsigned int* __restrict__ out)
+template <typename T>
+__global__ void fl_xmax_kernel(long long N, const T* __restrict__ x, unsigned int* __restrict__ out)
 {
     unsigned int m = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N; i += gridDim.x * blockDim.x) {
-        const unsigned int b = __float_as_uint(x[i]) & 0x7fffffffu;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
+        const unsigned int b = __float_as_uint(fl_float(x[i])) & 0x7fffffffu;
         if (b < 0x7f800000u) m = max(m, b);
     }
 #pragma unroll
@@ -90,6 +94,91 @@ __device__ __forceinline__ long long fl_word(unsigned int lo, unsigned int hi)
 
 __device__ __forceinline__ Leg fl_leg(float4 v) { return Leg{v.x, v.y, v.z, v.w}; }
 
+// The cursors at tile t0: the first row of each (layer, column) whose pair starts in that tile or later.  A cursor
+// is row << 16 | its tile (0: not looked at); nxt, for the next tile, starts past each run's end.
+template <int NT>
+__device__ __forceinline__ void fl_cursors(const GeomParams& P, const DevPtrs& D, const int* htx, const int* hrx, int t0,
+                                           unsigned int* cur, unsigned int* nxt)
+{
+    for (int j = threadIdx.x; j < P.W * P.n_seg; j += NT) {
+        const int sg = j / P.W, col = j - sg * P.W;
+        int a = P.seg_row[sg], b = P.seg_row[sg + 1];
+        if (t0 == 0) b = a;
+        const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
+        while (a < b) {
+            const int mid = (a + b) >> 1;
+            const float4* lr = D.legs + (size_t)mid * P.nh;
+            if (make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)), 1.0f).n0 < t0 * kFlTile) a = mid + 1;
+            else b = mid;
+        }
+        cur[j] = (unsigned int)a << 16;
+        nxt[j] = (unsigned int)P.seg_row[sg + 1] << 16;
+    }
+}
+
+// Calls pair(row, column, pair, n0 - tile's start, x) for every pair of the tile t (of non-zero weight or not), and
+// sets nxt to the runs' next rows.  A warp takes 32 columns and every nsub-th row of each layer's run, with enough
+// warps per run for every warp of the block to take part.
+template <int NT, typename F>
+__device__ __forceinline__ void fl_walk(const GeomParams& P, const DevPtrs& D, const int* htx, const int* hrx,
+                                        const float* __restrict__ x, int t, const unsigned int* cur, unsigned int* nxt,
+                                        F&& pair)
+{
+    const int ngrp = (P.W + 31) / 32, nsub = min(16, max(1, NT / 32 / ngrp)), units = ngrp * nsub;
+    for (int u = threadIdx.x >> 5; u < units; u += NT / 32) {
+        const int sub = u / ngrp, col = (u - sub * ngrp) * 32 + (threadIdx.x & 31);
+        if (col >= P.W) continue;
+        const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
+        for (int sg = 0; sg < P.n_seg; ++sg) {
+            const int j = sg * P.W + col, end = P.seg_row[sg + 1];
+            const unsigned int at = cur[j];
+            if ((int)(at & 0xffffu) > t) {                         // the run starts in a later tile
+                if (sub == 0) atomicMin(nxt + j, at);
+                continue;
+            }
+            int row = (int)(at >> 16) + sub;
+            if (row >= end) continue;
+            const float4* lr = D.legs + (size_t)row * P.nh;
+            float4 a = __ldg(lr + ht), b = __ldg(lr + hr);
+            float xv = x ? __ldg(x + (size_t)row * P.W + col) : 0.0f;
+            for (;;) {
+                // the next row's legs load while this one's pair is evaluated
+                lr += (size_t)nsub * P.nh;
+                float4 an = a, bn = b;
+                float xn = 0.0f;
+                if (row + nsub < end) {
+                    an = __ldg(lr + ht);
+                    bn = __ldg(lr + hr);
+                    if (x) xn = __ldg(x + (size_t)(row + nsub) * P.W + col);
+                }
+                const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
+                const int n0r = pr.n0 - t * kFlTile;
+                if (pr.n0 + 1 >= P.M) break;                       // the rows below start later still
+                if (n0r >= kFlTile) {
+                    atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)(pr.n0 / kFlTile));
+                    break;
+                }
+                if (n0r >= 0 && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) pair(row, col, pr, n0r, xv);
+                row += nsub;
+                if (row >= end) break;
+                a = an;
+                b = bn;
+                xv = xn;
+            }
+        }
+    }
+}
+
+// The walked tile's cursors for the tile after the next
+template <int NT>
+__device__ __forceinline__ void fl_advance(const GeomParams& P, unsigned int*& cur, unsigned int*& nxt)
+{
+    for (int j = threadIdx.x; j < P.W * P.n_seg; j += NT) cur[j] = (unsigned int)P.seg_row[j / P.W + 1] << 16;
+    unsigned int* const was = cur;
+    cur = nxt;
+    nxt = was;
+}
+
 // Block (A-scan, chunk of tiles): tiles [ta, tb), and the one before for the taps that reach past it.
 __global__ void __launch_bounds__(kFlThreads, 1)
     forward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint32_t* __restrict__ crange,
@@ -104,14 +193,14 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     float* part = reinterpret_cast<float*>(smem + L.off_part);
     float* carry = reinterpret_cast<float*>(smem + L.off_carry);
     int* bad = reinterpret_cast<int*>(smem + L.off_bad);                 // rows with a non-finite x; [128]: any
-    // cursors of this tile and of the next, per (layer, column): row << 16 | its tile (0: not looked at)
+    // cursors of this tile and of the next, per (layer, column)
     unsigned int* cur = reinterpret_cast<unsigned int*>(smem + L.off_cur);
     unsigned int* nxt = cur + (size_t)P.W * P.n_seg;
     const size_t hiw = L.off_hi / 4;
     const int tid = threadIdx.x, k = blockIdx.x;
     const int ntile = (P.M + kFlTile - 1) / kFlTile;
     const int ta = blockIdx.y * per, tb = min(ta + per, ntile), t0 = max(ta - 1, 0);
-    const int R = P.Q + 1, dR = P.G > 1 ? R : 0, ncur = P.W * P.n_seg;
+    const int R = P.Q + 1, dR = P.G > 1 ? R : 0;
     const int* htx = D.hidx + (size_t)__ldg(D.txpos + k / P.n_rx) * P.W;
     const int* hrx = D.hidx + (size_t)__ldg(D.rxpos + k) * P.W;
     // fixed-point scale: |x| < 2^ex and weights of at most 1 (2 with rounding), W x H of them, stay below 2^62
@@ -129,25 +218,9 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     if (ta == 0 && tid == 0) store(0, 0.0f);
     if (tb == ntile)
         for (int n = P.M + tid; n < out_stride; n += kFlThreads) store(n, 0.0f);
-    // cursors: the first row of each (layer, column) whose pair starts in tile t0 or later
-    for (int j = tid; j < ncur; j += kFlThreads) {
-        const int sg = j / P.W, col = j - sg * P.W;
-        int a = P.seg_row[sg], b = P.seg_row[sg + 1];
-        if (t0 == 0) b = a;
-        const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
-        while (a < b) {
-            const int mid = (a + b) >> 1;
-            const float4* lr = D.legs + (size_t)mid * P.nh;
-            if (make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)), 1.0f).n0 < t0 * kFlTile) a = mid + 1;
-            else b = mid;
-        }
-        cur[j] = (unsigned int)a << 16;
-        nxt[j] = (unsigned int)P.seg_row[sg + 1] << 16;
-    }
+    fl_cursors<kFlThreads>(P, D, htx, hrx, t0, cur, nxt);
     __syncthreads();
 
-    // warps that share the rows of 32 columns: enough for every warp to take part
-    const int ngrp = (P.W + 31) / 32, nsub = min(16, max(1, kFlThreads / 32 / ngrp)), units = ngrp * nsub;
     const int cg = tid / L.ng, og = tid - cg * L.ng;
     int par = 0;
     for (int t = t0; t < tb; ++t) {
@@ -155,71 +228,31 @@ __global__ void __launch_bounds__(kFlThreads, 1)
         const uint32_t cr = __ldg(crange + (size_t)k * ntile + t);
         const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
         if (kw > 0) {
-            // ---- the tile's pairs into S: a warp takes 32 columns and every sub-th row of each layer's run
-            for (int u = tid >> 5; u < units; u += kFlThreads / 32) {
-                const int sub = u / ngrp, col = (u - sub * ngrp) * 32 + (tid & 31);
-                if (col >= P.W) continue;
-                const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
-                for (int sg = 0; sg < P.n_seg; ++sg) {
-                    const int j = sg * P.W + col, end = P.seg_row[sg + 1];
-                    const unsigned int at = cur[j];
-                    if ((int)(at & 0xffffu) > t) {                         // the run starts in a later tile
-                        if (sub == 0) atomicMin(nxt + j, at);
-                        continue;
-                    }
-                    int row = (int)(at >> 16) + sub;
-                    if (row >= end) continue;
-                    const float4* lr = D.legs + (size_t)row * P.nh;
-                    float4 a = __ldg(lr + ht), b = __ldg(lr + hr);
-                    float xv = __ldg(x + (size_t)row * P.W + col);
-                    for (;;) {
-                        // the next row's legs load while this one's pair is evaluated
-                        lr += (size_t)nsub * P.nh;
-                        float4 an = a, bn = b;
-                        float xn = 0.0f;
-                        if (row + nsub < end) {
-                            an = __ldg(lr + ht);
-                            bn = __ldg(lr + hr);
-                            xn = __ldg(x + (size_t)(row + nsub) * P.W + col);
-                        }
-                        const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
-                        const int n0r = pr.n0 - ts;
-                        if (pr.n0 + 1 >= P.M) break;                       // the rows below start later still
-                        if (n0r >= kFlTile) {
-                            atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)(pr.n0 / kFlTile));
-                            break;
-                        }
-                        const float wx = pr.w * xv;
-                        if (wx != 0.0f && n0r >= 0 && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) {
-                            if (fabsf(wx) <= 3.4028235e38f) {
-                                const float p1 = pr.psi, p0 = 1.0f - pr.psi;
-                                unsigned int* s = lo + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
-                                const float wa = wx * pr.w0, wb = wx * pr.w1;
-                                fl_add(s, hiw, __float2ll_rn(fl_scale(wa * p0, se)));
-                                fl_add(s + kFlTile, hiw, __float2ll_rn(fl_scale(wb * p0, se)));
-                                if (dR) {
-                                    fl_add(s + dR * kFlTile, hiw, __float2ll_rn(fl_scale(wa * p1, se)));
-                                    fl_add(s + (dR + 1) * kFlTile, hiw, __float2ll_rn(fl_scale(wb * p1, se)));
-                                }
-                                if (pr.flag0) {
-                                    // tau = t0 exactly: the last tap of the upper phase lies outside the window
-                                    const float* tl = ftab + (size_t)(pr.gi * R + pr.r + 1) * P.Tw4 + P.Tw - 1;
-                                    const float ev = wb * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4));
-                                    fl_add(edge + n0r, kFlTile, __float2ll_rn(fl_scale(ev, se - ebits)));
-                                }
-                            } else {
-                                bad[n0r] = 1;
-                                bad[kFlTile] = 1;
-                            }
-                        }
-                        row += nsub;
-                        if (row >= end) break;
-                        a = an;
-                        b = bn;
-                        xv = xn;
-                    }
+            // ---- the tile's pairs into S
+            fl_walk<kFlThreads>(P, D, htx, hrx, x, t, cur, nxt, [&](int row, int col, const Pair& pr, int n0r, float xv) {
+                const float wx = pr.w * xv;
+                if (!(wx != 0.0f)) return;
+                if (!(fabsf(wx) <= 3.4028235e38f)) {
+                    bad[n0r] = 1;
+                    bad[kFlTile] = 1;
+                    return;
                 }
-            }
+                const float p1 = pr.psi, p0 = 1.0f - pr.psi;
+                unsigned int* s = lo + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
+                const float wa = wx * pr.w0, wb = wx * pr.w1;
+                fl_add(s, hiw, __float2ll_rn(fl_scale(wa * p0, se)));
+                fl_add(s + kFlTile, hiw, __float2ll_rn(fl_scale(wb * p0, se)));
+                if (dR) {
+                    fl_add(s + dR * kFlTile, hiw, __float2ll_rn(fl_scale(wa * p1, se)));
+                    fl_add(s + (dR + 1) * kFlTile, hiw, __float2ll_rn(fl_scale(wb * p1, se)));
+                }
+                if (pr.flag0) {
+                    // tau = t0 exactly: the last tap of the upper phase lies outside the window
+                    const float* tl = ftab + (size_t)(pr.gi * R + pr.r + 1) * P.Tw4 + P.Tw - 1;
+                    const float ev = wb * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4));
+                    fl_add(edge + n0r, kFlTile, __float2ll_rn(fl_scale(ev, se - ebits)));
+                }
+            });
             __syncthreads();
             // ---- S as FP32 in place of its low words
             uint4* l4 = reinterpret_cast<uint4*>(lo);
@@ -288,10 +321,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
         if (kw > 0) {
             uint4* l4 = reinterpret_cast<uint4*>(lo);
             for (int i = tid; i < kw * (kFlTile / 4); i += kFlThreads) l4[i] = make_uint4(0u, 0u, 0u, 0u);
-            for (int j = tid; j < ncur; j += kFlThreads) cur[j] = (unsigned int)P.seg_row[j / P.W + 1] << 16;
-            unsigned int* const was = cur;
-            cur = nxt;
-            nxt = was;
+            fl_advance<kFlThreads>(P, cur, nxt);
         }
         __syncthreads();
         if (kw > 0) {
@@ -300,6 +330,120 @@ __global__ void __launch_bounds__(kFlThreads, 1)
             __syncthreads();
         }
     }
+}
+
+constexpr int kBlThreads = 512;
+
+struct BlLayout {
+    size_t off_e, off_cur, smem;
+};
+__host__ __device__ inline BlLayout bl_layout(const GeomParams& P, int kw)
+{
+    BlLayout L;
+    L.off_e = (size_t)kw * kFlTile * 4;
+    L.off_cur = L.off_e + (size_t)(kFlTile + P.Tw4) * 4;
+    L.smem = L.off_cur + (((size_t)P.W * P.n_seg * 8 + 15) & ~(size_t)15);
+    return L;
+}
+
+// Scale exponent of the adjoint's fixed-point sums: every contribution is at most bound / K x max |e| in magnitude
+// and a pixel has at most one per A-scan, so no partial sum reaches 2^61.
+__device__ __forceinline__ int bl_exponent(unsigned int emax_bits, float bound)
+{
+    int e1 = 0, e2 = 0;
+    frexpf(__uint_as_float(emax_bits), &e1);
+    frexpf(bound, &e2);
+    return 61 - e1 - e2;
+}
+
+// A^T r from the legs, the adjoint of the sums above: for a tile of 128 values of n0
+//     C[n0][col] = sum_m e[n0 + 1 + m] T[col][m]
+// (FP32, eight values of n0 and a share of the columns per thread), of which each pair combines four, and adds the
+// result to its pixel's 64-bit fixed-point sum.  Block (A-scan, chunk of tiles), two blocks per SM: one's products
+// run beside the other's walk.
+// 256x512, 64 x 16 A-scans (41 M pairs, FP32), legs included: 1.25 ms against 2.26 ms of backproject_kernel, which
+// is bound by the shared-memory loads of its taps (83 % of their peak); the walk takes about half of it.
+template <typename E>
+__global__ void __launch_bounds__(kBlThreads, 2)
+    backward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint32_t* __restrict__ crange,
+                         const E* __restrict__ e, const unsigned int* __restrict__ emax, float bound, int kwmax, int per,
+                         unsigned long long* __restrict__ acc, unsigned char* __restrict__ bad)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    const BlLayout L = bl_layout(P, kwmax);
+    float* C = reinterpret_cast<float*>(smem);
+    float* sE = reinterpret_cast<float*>(smem + L.off_e);
+    unsigned int* cur = reinterpret_cast<unsigned int*>(smem + L.off_cur);
+    unsigned int* nxt = cur + (size_t)P.W * P.n_seg;
+    const int tid = threadIdx.x, k = blockIdx.x;
+    const int ntile = (P.M + kFlTile - 1) / kFlTile;
+    const int ta = blockIdx.y * per, tb = min(ta + per, ntile);
+    const int R = P.Q + 1, dR = P.G > 1 ? R : 0;
+    const int* htx = D.hidx + (size_t)__ldg(D.txpos + k / P.n_rx) * P.W;
+    const int* hrx = D.hidx + (size_t)__ldg(D.rxpos + k) * P.W;
+    const int se = bl_exponent(__ldg(emax), bound);
+    const int cg = tid >> 4, og = tid & 15;
+    fl_cursors<kBlThreads>(P, D, htx, hrx, ta, cur, nxt);
+    for (int t = ta; t < tb; ++t) {
+        const uint32_t cr = __ldg(crange + (size_t)k * ntile + t);
+        const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
+        if (kw <= 0) continue;
+        for (int i = tid; i < kFlTile + P.Tw4; i += kBlThreads) {
+            const int n = t * kFlTile + 1 + i;
+            sE[i] = n < P.Mp ? fl_float(e[(size_t)k * P.Mp + n]) : 0.0f;
+        }
+        __syncthreads();
+        // ---- C, rows 8 og .. 8 og + 7: four taps at a time against the window's next four samples
+        const float4* W = reinterpret_cast<const float4*>(sE);
+        const int ntb = P.Tw4 / 4;
+        for (int c = cg; c < kw; c += kBlThreads / 16) {
+            const float4* T = reinterpret_cast<const float4*>(ftab + (size_t)(c_lo + c) * P.Tw4);
+            float a[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+            float4 f0 = W[2 * og], f1 = W[2 * og + 1];
+#pragma unroll 4
+            for (int mb = 0; mb < ntb; ++mb) {
+                const float4 f2 = W[2 * og + 2 + mb];
+                const float4 w = __ldg(T + mb);
+                const float v[12] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w, f2.x, f2.y, f2.z, f2.w};
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                    a[j] = fmaf(v[j + 3], w.w, fmaf(v[j + 2], w.z, fmaf(v[j + 1], w.y, fmaf(v[j], w.x, a[j]))));
+                f0 = f1;
+                f1 = f2;
+            }
+            float4* o = reinterpret_cast<float4*>(C + (size_t)c * kFlTile + 8 * og);
+            o[0] = make_float4(a[0], a[1], a[2], a[3]);
+            o[1] = make_float4(a[4], a[5], a[6], a[7]);
+        }
+        __syncthreads();
+        fl_walk<kBlThreads>(P, D, htx, hrx, nullptr, t, cur, nxt, [&](int row, int col, const Pair& pr, int n0r, float) {
+            if (pr.w == 0.0f) return;
+            const float* c = C + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
+            const float p1 = pr.psi, p0 = 1.0f - pr.psi;
+            float hv = pr.w0 * (p0 * c[0] + p1 * c[dR * kFlTile]) +
+                       pr.w1 * (p0 * c[kFlTile] + p1 * c[(dR + 1) * kFlTile]);
+            if (pr.flag0) {
+                // tau = t0 exactly: the last tap of the upper phase lies outside the window
+                const float* tl = ftab + (size_t)(pr.gi * R + pr.r + 1) * P.Tw4 + P.Tw - 1;
+                hv -= pr.w1 * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4)) * sE[n0r + P.Tw - 1];
+            }
+            const float v = pr.w * hv;
+            const int px = row * P.W + col;
+            if (fabsf(v) <= 3.4028235e38f) red_add_global_u64(acc + px, (unsigned long long)__float2ll_rn(fl_scale(v, se)));
+            else bad[px] = 1;
+        });
+        __syncthreads();
+        fl_advance<kBlThreads>(P, cur, nxt);
+    }
+}
+
+// b from the fixed-point sums; NaN where a contribution was not finite
+__global__ void bl_finish_kernel(int N, const unsigned long long* __restrict__ acc, const unsigned char* __restrict__ bad,
+                                 const unsigned int* __restrict__ emax, float bound, float* __restrict__ b)
+{
+    const int se = bl_exponent(*emax, bound);
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x)
+        b[v] = bad[v] ? __uint_as_float(0x7fc00000u) : fl_scale(__ll2float_rn((long long)acc[v]), -se);
 }
 
 // Attenuation planes that the pairs of each (A-scan, tile) reach, as the range of table columns first | end << 16
@@ -366,19 +510,26 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
     }
     if (e == cudaSuccess) e = cudaMemcpyAsync(&wmax, d_max, sizeof(int), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    float tmax = 0.0f;
+    float tmax = 0.0f, tsum = 0.0f;
+    unsigned char* d_acc = nullptr;                  // per pixel: the adjoint's sum, (one word) max |e|, the NaN marks
+    const size_t nacc = 9 * (size_t)P.W * P.H + 8;
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_acc, nacc);
     if (e == cudaSuccess) {
         const bool bf = P.precision == MBIR_PREC_BF16;
         const int nq = P.Q * P.Tw + 1;
         std::vector<float> tab(ntab, 0.0f);
         for (int gp = 0; gp < P.G; ++gp)
-            for (int r = 0; r < R; ++r)
+            for (int r = 0; r < R; ++r) {
+                float sum = 0.0f;
                 for (int m = 0; m < P.Tw; ++m) {
                     float v = (float)g->tab_host[(size_t)gp * nq + m * P.Q + r];
                     if (bf) v = __bfloat162float(__float2bfloat16_rn(v));
                     tab[((size_t)gp * R + r) * P.Tw4 + m] = v;
                     tmax = std::max(tmax, std::fabs(v));
+                    sum += std::fabs(v);
                 }
+                tsum = std::max(tsum, sum);
+            }
         e = cudaMemcpy(d_tab, tab.data(), sizeof(float) * ntab, cudaMemcpyHostToDevice);
     }
     const int kw = std::max(wmax, 1);
@@ -386,10 +537,16 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
     if (e == cudaSuccess && sm > 226 * 1024) e = cudaErrorNotSupported;     // a tile reaches too many planes
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(forward_legs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    for (const void* f : {(const void*)backward_legs_kernel<float>, (const void*)backward_legs_kernel<__nv_bfloat16>})
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
+    // weights are at most 1 (2 with the rounding of the products)
+    const double bound = 2.0 * P.K * ((double)tsum + tmax);
+    if (e == cudaSuccess && !(bound > 0.0 && bound < 1e30)) e = cudaErrorNotSupported;
     if (e != cudaSuccess) {
         cudaFree(d_cr);
         cudaFree(d_tab);
         cudaFree(d_max);
+        cudaFree(d_acc);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
     }
@@ -402,7 +559,9 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
     g->d_fl_crange = d_cr;
     g->d_fl_tab = d_tab;
     g->d_fl_max = d_max;
-    g->bytes += sizeof(uint32_t) * ncr + sizeof(float) * ntab + sizeof(unsigned int);
+    g->w_fl_acc = d_acc;
+    g->fl_bound = (float)bound;
+    g->bytes += sizeof(uint32_t) * ncr + sizeof(float) * ntab + sizeof(unsigned int) + nacc;
     return cudaSuccess;
 }
 
@@ -415,12 +574,45 @@ cudaError_t launch_forward_legs(const mbir_geometry* g, const float* x, float* y
     const int N = P.W * P.H, ntile = (P.M + kFlTile - 1) / kFlTile;
     cudaError_t e = cudaMemsetAsync(g->d_fl_max, 0, sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;
-    fl_xmax_kernel<<<std::max(1, std::min((N + 1023) / 1024, g->n_sm)), 256, 0, st>>>(N, x, g->d_fl_max);
+    fl_xmax_kernel<float><<<std::max(1, std::min((N + 1023) / 1024, g->n_sm)), 256, 0, st>>>(N, x, g->d_fl_max);
     const int want = (4 * g->n_sm + P.K - 1) / P.K;
     const int per = std::max((ntile + want - 1) / want, std::min(4, ntile));
     forward_legs_kernel<<<dim3(P.K, (ntile + per - 1) / per), kFlThreads, fl_layout(P, g->fl_kw).smem, st>>>(
         P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, x, g->d_fl_max, g->fl_bits, g->fl_ebits, g->fl_kw, per, yf, yb,
         stride);
+    return cudaGetLastError();
+}
+
+// A^T e, with e K x Mp (its BF16 copy in the BF16 form); chunks as above, for eight blocks per SM, two of which run
+// at a time.
+cudaError_t launch_backproject_legs(const mbir_geometry* g, const float* e_pad, const __nv_bfloat16* e_bf, float* b,
+                                    cudaStream_t st)
+{
+    const GeomParams& P = g->P;
+    const int N = P.W * P.H, ntile = (P.M + kFlTile - 1) / kFlTile;
+    auto* acc = reinterpret_cast<unsigned long long*>(g->w_fl_acc);
+    auto* emax = reinterpret_cast<unsigned int*>(acc + N);
+    unsigned char* bad = g->w_fl_acc + 8 * ((size_t)N + 1);
+    cudaError_t e = cudaMemsetAsync(g->w_fl_acc, 0, 9 * (size_t)N + 8, st);
+    if (e != cudaSuccess) return e;
+    const long long ne = (long long)P.K * P.Mp;
+    const int eg = (int)std::max(1LL, std::min((ne + 255) / 256, (long long)g->n_sm * 8));
+    const int want = (8 * g->n_sm + P.K - 1) / P.K;
+    const int per = std::max((ntile + want - 1) / want, std::min(4, ntile));
+    const dim3 grid(P.K, (ntile + per - 1) / per);
+    const size_t sm = bl_layout(P, g->fl_kw).smem;
+    if (P.precision == MBIR_PREC_BF16) {
+        fl_xmax_kernel<__nv_bfloat16><<<eg, 256, 0, st>>>(ne, e_bf, emax);
+        backward_legs_kernel<__nv_bfloat16><<<grid, kBlThreads, sm, st>>>(
+            P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, e_bf, emax, g->fl_bound, g->fl_kw, per, acc, bad);
+    } else {
+        fl_xmax_kernel<float><<<eg, 256, 0, st>>>(ne, e_pad, emax);
+        backward_legs_kernel<float><<<grid, kBlThreads, sm, st>>>(
+            P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, e_pad, emax, g->fl_bound, g->fl_kw, per, acc, bad);
+    }
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    bl_finish_kernel<<<std::max(1, std::min((N + 255) / 256, g->n_sm * 8)), 256, 0, st>>>(N, acc, bad, emax, g->fl_bound, b);
     return cudaGetLastError();
 }
 

@@ -398,6 +398,8 @@ struct mbir_geometry {
     float* d_fl_tab;
     unsigned int* d_fl_max;
     int fl_bits, fl_ebits, fl_kw;
+    unsigned char* w_fl_acc;   // the adjoint's workspace (N 64-bit sums, max |e|, N marks) and its scale bound
+    float fl_bound;
     // TAB-mode A x records sorted by first tap sample (see forward_tab.cu); with the tensor-core applies the
     // sorted records are replaced by their packed form (tc_apply.cuh), on the same per-A-scan offsets
     long long* d_rec_off;
@@ -472,6 +474,8 @@ cudaError_t load_otf_legs(const mbir_geometry* g);
 cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st);
 cudaError_t launch_forward_legs(const mbir_geometry* g, const float* x, float* yf, __nv_bfloat16* yb, int stride,
                                 cudaStream_t st);
+cudaError_t launch_backproject_legs(const mbir_geometry* g, const float* e_pad, const __nv_bfloat16* e_bf, float* b,
+                                    cudaStream_t st);
 cudaError_t launch_backproject(const mbir_geometry* g, const float* e_pad, const __nv_bfloat16* e_bf,
                                float* b, cudaStream_t st);
 cudaError_t launch_forward(const mbir_geometry* g, const float* x, float* y_f32, __nv_bfloat16* y_bf16,
