@@ -433,9 +433,9 @@ def run_gpu(args):
 
     # per iteration: A^T r (tensor cores: the previous step's residual update with max |e|, the pool, the
     # fixed-point sums into b; CUDA cores: the residual update, the partial images and their reduction), the
-    # prior stencil with the previous step's image update, PR+ scalars, direction, A x, projection, step; per
-    # reconstruction the projection of y and the residual's sum of squares first, the last image update after
-    per_iter = 3 + 6
+    # prior stencil with the previous step's image update and the PR+ scalars, direction, A x, projection with the
+    # step; per reconstruction the projection of y and the residual's sum of squares first, the last image update after
+    per_iter = 3 + 4
     launches = args.steps * (per_iter * scene.n_iter + 3)
 
     out = {"metric": "recons/s", "value": value, "unit": "recons/s", "n_gpus": world, "steps": args.steps,

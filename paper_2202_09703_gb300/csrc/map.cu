@@ -17,6 +17,30 @@
 
 namespace mbir {
 
+// Polak-Ribiere+ coefficient with a descent restart
+__device__ __forceinline__ void finalize_dir(const double* part, int nb, int it, double* sc, double* gnorm_hist, double* sh)
+{
+    double a0 = 0, a1 = 0, a2 = 0;
+    for (int t = threadIdx.x; t < nb; t += blockDim.x) {
+        a0 += __ldcg(part + 3 * t);
+        a1 += __ldcg(part + 3 * t + 1);
+        a2 += __ldcg(part + 3 * t + 2);
+    }
+    double gg = block_sum(a0, sh), ggp = block_sum(a1, sh), gdp = block_sum(a2, sh);
+    if (threadIdx.x == 0) {
+        double beta = 0.0;
+        if (it > 0 && sc[S_GGPREV] > 0.0) beta = fmax((gg - ggp) / sc[S_GGPREV], 0.0);
+        double gd = -gg + beta * gdp;
+        if (!(gd < 0.0)) { beta = 0.0; gd = -gg; }
+        sc[S_GG] = gg;
+        sc[S_BETA] = beta;
+        sc[S_GD] = gd;
+        sc[S_GGPREV] = gg;
+        if (!isfinite(gg)) sc[S_BAD] = 1.0;
+        if (gnorm_hist) gnorm_hist[it] = sqrt(gg);
+    }
+}
+
 // The MAP update and the prior stencil in one pass: with dupd given, x is first moved by the previous
 // iteration's step, x + alpha dupd (alpha = sc[S_ALPHA]), at the pixel and at its eight neighbours, and the
 // moved image is written to xout; then grad = -b/sigma^2 + grad R(x) at the moved image, with FP64 partials
@@ -24,8 +48,8 @@ namespace mbir {
 __global__ void grad_kernel(GeomParams P, PriorParams pr, const float* __restrict__ x, const float* __restrict__ b,
                             const float* __restrict__ msq, const float* __restrict__ gprev,
                             const float* __restrict__ dprev, float* __restrict__ grad, double* __restrict__ part,
-                            int with_data, const float* __restrict__ dupd, const double* __restrict__ sc,
-                            float* __restrict__ xout)
+                            int with_data, const float* __restrict__ dupd, double* __restrict__ sc,
+                            float* __restrict__ xout, int it, double* __restrict__ hist)
 {
     __shared__ double sh[32];
     const int N = P.W * P.H;
@@ -61,6 +85,8 @@ __global__ void grad_kernel(GeomParams P, PriorParams pr, const float* __restric
         part[3 * blockIdx.x + 1] = s1;
         part[3 * blockIdx.x + 2] = s2;
     }
+    if (hist && last_block(reinterpret_cast<unsigned int*>(sc + S_TICKETS)))
+        finalize_dir(part, gridDim.x, it, sc, hist, sh);
 }
 
 // xout = xin + alpha d (alpha = sc[S_ALPHA]); in place when xout == xin
@@ -69,32 +95,6 @@ __global__ void x_step_kernel(int N, const double* __restrict__ sc, const float*
 {
     const float a = (float)sc[S_ALPHA];
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < N; t += gridDim.x * blockDim.x) xout[t] = fmaf(a, d[t], xin[t]);
-}
-
-// Polak-Ribiere+ coefficient with a descent restart
-__global__ void finalize_dir_kernel(const double* __restrict__ part, int nb, int it, double* __restrict__ sc,
-                                    double* __restrict__ gnorm_hist)
-{
-    __shared__ double sh[32];
-    double a0 = 0, a1 = 0, a2 = 0;
-    for (int t = threadIdx.x; t < nb; t += blockDim.x) {
-        a0 += part[3 * t];
-        a1 += part[3 * t + 1];
-        a2 += part[3 * t + 2];
-    }
-    double gg = block_sum(a0, sh), ggp = block_sum(a1, sh), gdp = block_sum(a2, sh);
-    if (threadIdx.x == 0) {
-        double beta = 0.0;
-        if (it > 0 && sc[S_GGPREV] > 0.0) beta = fmax((gg - ggp) / sc[S_GGPREV], 0.0);
-        double gd = -gg + beta * gdp;
-        if (!(gd < 0.0)) { beta = 0.0; gd = -gg; }
-        sc[S_GG] = gg;
-        sc[S_BETA] = beta;
-        sc[S_GD] = gd;
-        sc[S_GGPREV] = gg;
-        if (!isfinite(gg)) sc[S_BAD] = 1.0;
-        if (gnorm_hist) gnorm_hist[it] = sqrt(gg);
-    }
 }
 
 // d = -grad + beta dprev; gprev = grad; partial of sum b kappa(x_s - x_r) (d_s - d_r)^2
@@ -132,13 +132,34 @@ __global__ void dir_kernel(GeomParams P, PriorParams pr, const float* __restrict
     if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
+// The step alpha along d from the rows' |q|^2 and the blocks' prior curvature
+__device__ __forceinline__ void finalize_step(const double* qpart, int nq, const double* __restrict__ cpart, int nc,
+                                              float inv_s2, double* sc, double* sh)
+{
+    double a = 0, b = 0;
+    for (int t = threadIdx.x; t < nq; t += blockDim.x) a += __ldcg(qpart + t);
+    for (int t = threadIdx.x; t < nc; t += blockDim.x) b += cpart[t];
+    double qq = block_sum(a, sh), cv = block_sum(b, sh);
+    if (threadIdx.x == 0) {
+        double den = qq * (double)inv_s2 + cv;
+        double alpha = den > 0.0 ? -sc[S_GD] / den : 0.0;
+        if (!isfinite(alpha)) { alpha = 0.0; sc[S_BAD] = 1.0; }
+        sc[S_QQ] = qq;
+        sc[S_CURV] = cv;
+        sc[S_ALPHA] = alpha;
+    }
+}
+
 // Per A-scan direct-arrival projection (eq. 1): g = <d,r>/|d|^2, out = r - g d.
 // src rows of stride `sin` (float or bf16, optional subtraction of `sub`),
 // dst rows of stride `sout` padded with zeros; FP64 partial |out|^2 per row.
+// With sc given, the last row to finish takes the step (finalize_step, with
+// the nc curvature partials cpart), which saves a launch as in grad_kernel.
 __global__ void project_kernel(GeomParams P, const void* __restrict__ src, int src_bf16, int sin,
                                const float* __restrict__ sub, int ssub, const float* __restrict__ direct,
                                const float* __restrict__ dinv, int use_direct, float* __restrict__ dst, int sout,
-                               float* __restrict__ gk, double* __restrict__ part)
+                               float* __restrict__ gk, double* __restrict__ part, const double* __restrict__ cpart,
+                               int nc, float inv_s2, double* __restrict__ sc)
 {
     __shared__ double sh[32];
     const int k = blockIdx.x;
@@ -171,24 +192,8 @@ __global__ void project_kernel(GeomParams P, const void* __restrict__ src, int s
         if (gk) gk[k] = g;
         if (part) part[k] = e2;
     }
-}
-
-__global__ void finalize_step_kernel(const double* __restrict__ qpart, int nq, const double* __restrict__ cpart,
-                                     int nc, float inv_s2, double* __restrict__ sc)
-{
-    __shared__ double sh[32];
-    double a = 0, b = 0;
-    for (int t = threadIdx.x; t < nq; t += blockDim.x) a += qpart[t];
-    for (int t = threadIdx.x; t < nc; t += blockDim.x) b += cpart[t];
-    double qq = block_sum(a, sh), cv = block_sum(b, sh);
-    if (threadIdx.x == 0) {
-        double den = qq * (double)inv_s2 + cv;
-        double alpha = den > 0.0 ? -sc[S_GD] / den : 0.0;
-        if (!isfinite(alpha)) { alpha = 0.0; sc[S_BAD] = 1.0; }
-        sc[S_QQ] = qq;
-        sc[S_CURV] = cv;
-        sc[S_ALPHA] = alpha;
-    }
+    if (sc && last_block(reinterpret_cast<unsigned int*>(sc + S_TICKETS) + 1))
+        finalize_step(part, gridDim.x, cpart, nc, inv_s2, sc, sh);
 }
 
 // x += alpha d (first N threads), e -= alpha q (next K*Mp), optional BF16 copy
@@ -509,10 +514,10 @@ int reconstruct_core(mbir_geometry* g, const void* y_dev, int y_bf16, const mbir
     if (x_given) {
         CK(launch_forward(g, x, g->w_q, nullptr, P.Mp, st));
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, y_dev, y_bf16, P.M, g->w_q, P.Mp, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_e, P.Mp, nullptr, part);
+                                                    use_direct, g->w_e, P.Mp, nullptr, part, nullptr, 0, 0.0f, nullptr);
     } else {
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, y_dev, y_bf16, P.M, nullptr, 0, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_e, P.Mp, nullptr, part);
+                                                    use_direct, g->w_e, P.Mp, nullptr, part, nullptr, 0, 0.0f, nullptr);
     }
     CK(cudaGetLastError());
     residual_sum_kernel<<<1, kRedThreads, 0, st>>>(part, P.K, sc);
@@ -546,17 +551,16 @@ int reconstruct_core(mbir_geometry* g, const void* y_dev, int y_bf16, const mbir
         }
         prof_end(g, st);
         grad_kernel<<<nbpix, kRedThreads, 0, st>>>(P, pp, xc, g->w_b, g->w_msq, g->w_gprev, dcur, g->w_grad, part, 1,
-                                                   pending ? dcur : nullptr, sc, xo);
+                                                   pending ? dcur : nullptr, sc, xo, it, g->w_hist + g->hist_len);
         if (pending) std::swap(xc, xo);
-        finalize_dir_kernel<<<1, kRedThreads, 0, st>>>(part, nbpix, it, sc, g->w_hist + g->hist_len);
         dir_kernel<<<nbpix, kRedThreads, 0, st>>>(P, pp, xc, g->w_grad, dcur, g->w_msq, sc, dnxt, g->w_gprev, part2);
         CK(cudaGetLastError());
         prof_begin(g, 0, st);
         CK(launch_forward(g, dnxt, g->w_q, nullptr, P.Mp, st));
         prof_end(g, st);
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, g->w_q, 0, P.Mp, nullptr, 0, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_q, P.Mp, nullptr, part);
-        finalize_step_kernel<<<1, kRedThreads, 0, st>>>(part, P.K, part2, nbpix, pp.inv_s2, sc);
+                                                    use_direct, g->w_q, P.Mp, nullptr, part, part2, nbpix,
+                                                    pp.inv_s2, sc);
         if (fuse) {
             pending = true;
         } else {
@@ -575,7 +579,7 @@ int reconstruct_core(mbir_geometry* g, const void* y_dev, int y_bf16, const mbir
     if (g_dev) {
         CK(launch_forward(g, x, g->w_q, nullptr, P.Mp, st));
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, y_dev, y_bf16, P.M, g->w_q, P.Mp, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_q, P.Mp, g_dev, nullptr);
+                                                    use_direct, g->w_q, P.Mp, g_dev, nullptr, nullptr, 0, 0.0f, nullptr);
         CK(cudaGetLastError());
     }
     std::vector<double> scal(S_COUNT);
@@ -642,10 +646,10 @@ int icd_core(mbir_geometry* g, const void* y_dev, int y_bf16, const mbir_prior* 
     if (x_given) {
         CK(launch_forward(g, x, g->w_q, nullptr, P.Mp, st));
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, y_dev, y_bf16, P.M, g->w_q, P.Mp, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_e, P.Mp, nullptr, part);
+                                                    use_direct, g->w_e, P.Mp, nullptr, part, nullptr, 0, 0.0f, nullptr);
     } else {
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, y_dev, y_bf16, P.M, nullptr, 0, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_e, P.Mp, nullptr, part);
+                                                    use_direct, g->w_e, P.Mp, nullptr, part, nullptr, 0, 0.0f, nullptr);
     }
     CK(cudaGetLastError());
     residual_sum_kernel<<<1, kRedThreads, 0, st>>>(part, P.K, sc);
@@ -683,7 +687,7 @@ int icd_core(mbir_geometry* g, const void* y_dev, int y_bf16, const mbir_prior* 
             if (e != cudaSuccess) return e;
             prof_end(g, s);
             project_kernel<<<P.K, kRedThreads, 0, s>>>(P, g->w_q, 0, P.Mp, nullptr, 0, g->d_direct, g->d_dinv,
-                                                       use_direct, g->w_q, P.Mp, nullptr, part2);
+                                                       use_direct, g->w_q, P.Mp, nullptr, part2, nullptr, 0, 0.0f, nullptr);
             icd_step_kernel<<<1, kRedThreads, 0, s>>>(part, nbpix, part2, P.K, pp.inv_s2, sc);
             update_kernel<<<ublocks, 256, 0, s>>>(N, KMp, sc, x, dx, g->w_e, g->w_q, ebf);
             if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -733,7 +737,7 @@ int icd_core(mbir_geometry* g, const void* y_dev, int y_bf16, const mbir_prior* 
     if (g_dev) {
         CK(launch_forward(g, x, g->w_q, nullptr, P.Mp, st));
         project_kernel<<<P.K, kRedThreads, 0, st>>>(P, y_dev, y_bf16, P.M, g->w_q, P.Mp, g->d_direct, g->d_dinv,
-                                                    use_direct, g->w_q, P.Mp, g_dev, nullptr);
+                                                    use_direct, g->w_q, P.Mp, g_dev, nullptr, nullptr, 0, 0.0f, nullptr);
         CK(cudaGetLastError());
     }
     std::vector<double> scal(S_COUNT);
@@ -822,7 +826,7 @@ int mbir_project(const mbir_geometry* g, const float* r_dev, float* e_dev, float
     // rows are processed one block each; in-place use is safe (a block reads
     // its row fully before writing it)
     project_kernel<<<g->P.K, kRedThreads, 0, st>>>(g->P, r_dev, 0, g->P.M, nullptr, 0, g->d_direct, g->d_dinv, 1,
-                                                   e_dev, g->P.M, gk_dev, nullptr);
+                                                   e_dev, g->P.M, gk_dev, nullptr, nullptr, 0, 0.0f, nullptr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? MBIR_OK : cerr_code(e);
 }
@@ -851,7 +855,7 @@ int mbir_prior_gradient(const mbir_geometry* gc, const mbir_prior* pr, const flo
     const int nb = (N + kRedThreads - 1) / kRedThreads;
     CK(cudaMemsetAsync(g->w_gprev, 0, sizeof(float) * N, st));
     grad_kernel<<<nb, kRedThreads, 0, st>>>(g->P, prior_params(&tmp), x_dev, nullptr, g->w_msq, g->w_gprev,
-                                           g->w_gprev, out_dev, g->w_part, 0, nullptr, nullptr, nullptr);
+                                           g->w_gprev, out_dev, g->w_part, 0, nullptr, nullptr, nullptr, 0, nullptr);
     cudaError_t e = cudaGetLastError();
     return e == cudaSuccess ? MBIR_OK : cerr_code(e);
 }
@@ -948,7 +952,7 @@ cudaError_t launch_project_rows(const mbir_geometry* g, const void* src, int src
                                 int ssub, float* dst, int sout, float* gk, double* part, cudaStream_t st)
 {
     project_kernel<<<g->P.K, kRedThreads, 0, st>>>(g->P, src, src_bf16, sin, sub, ssub, g->d_direct, g->d_dinv, 1,
-                                                   dst, sout, gk, part);
+                                                   dst, sout, gk, part, nullptr, 0, 0.0f, nullptr);
     return cudaGetLastError();
 }
 

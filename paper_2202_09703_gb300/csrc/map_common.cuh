@@ -18,6 +18,7 @@ struct PriorParams {
 // scalar slots (doubles)
 enum {
     S_GG = 0, S_GGP, S_GDP, S_GGPREV, S_BETA, S_GD, S_QQ, S_CURV, S_ALPHA, S_EE, S_PRIOR, S_BAD,
+    S_TICKETS,             // two block counters (last_block) of grad_kernel and project_kernel
     S_COUNT = 16
 };
 
@@ -33,6 +34,20 @@ __device__ __forceinline__ double block_sum(double v, double* sh)
     if (threadIdx.x == 0)
         for (int w = 0; w < (int)(blockDim.x >> 5); ++w) r += sh[w];
     return r;   // valid in thread 0
+}
+
+// True in every thread of the block that calls this last, which then sees what all blocks wrote before their
+// calls (thread 0's writes); `ticket` starts at zero and is left at zero.
+__device__ __forceinline__ bool last_block(unsigned int* ticket)
+{
+    __shared__ bool last;
+    if (threadIdx.x == 0) {
+        __threadfence();
+        last = atomicInc(ticket, gridDim.x - 1) == gridDim.x - 1;
+        __threadfence();
+    }
+    __syncthreads();
+    return last;
 }
 
 // QGGMRF potential (eq. 15) and its derivatives, in FP32 through log2/exp2.

@@ -421,7 +421,7 @@ struct mbir_geometry {
     // tensor-core A^T (see tc_adjoint.cu, tc_stream.cuh)
     unsigned long long* w_tc_acc;   // per pixel: fixed-point sum, N + 1 (the last word: bits of max |e|)
     float tc_bound;        // scale bound of the fixed-point sums (build_tc_adjoint)
-    int* d_tc_counter;
+    int* d_tc_counter;     // in w_tc_acc, after its max |e| word
     // tensor-core A x (see tc_stream.cuh, tc_fwd_stream.cu)
     mbir::TsView* d_tf_view;   // fwd_tcs_kernel's view without the per-call fields (device memory)
     mbir::TbView* d_tb_view;   // bwd_tcs_kernel's view without the residual (device memory)

@@ -88,10 +88,8 @@ cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
     if (!g->d_tb_key || g->n_records <= 0) return cudaErrorNotSupported;
     const int N = P.W * P.H;
     unsigned long long* d_acc = nullptr;
-    int* d_ctr = nullptr;
-    cudaError_t e = cudaMalloc((void**)&d_acc, sizeof(unsigned long long) * ((size_t)N + 1));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_ctr, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_acc, 0, sizeof(unsigned long long) * ((size_t)N + 1), st);
+    cudaError_t e = cudaMalloc((void**)&d_acc, sizeof(unsigned long long) * ((size_t)N + 2));
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_acc, 0, sizeof(unsigned long long) * ((size_t)N + 2), st);
     unsigned int wbits = 0;
     if (e == cudaSuccess) {
         unsigned int* d_wmax = reinterpret_cast<unsigned int*>(d_acc + N);
@@ -122,24 +120,21 @@ cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
     const double bound = 2.0 * P.K * (double)wmax * (tsum + tmax);
     if (e == cudaSuccess && !(bound > 0.0 && bound < 1e30)) e = cudaErrorNotSupported;
     if (e != cudaSuccess) {
-        void* ptrs[] = {d_acc, d_ctr};
-        for (void* p : ptrs) cudaFree(p);
+        cudaFree(d_acc);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
     }
     g->w_tc_acc = d_acc;
-    g->d_tc_counter = d_ctr;
+    g->d_tc_counter = reinterpret_cast<int*>(d_acc + N + 1);
     g->tc_bound = (float)bound;
-    g->bytes += sizeof(int) + sizeof(unsigned long long) * ((size_t)N + 1);
+    g->bytes += sizeof(unsigned long long) * ((size_t)N + 2);
     return cudaSuccess;
 }
 
 // The tables above, freed when the tensor-core A^T is not used after all.
 void free_tc_adjoint(mbir_geometry* g)
 {
-    void* ptrs[] = {g->w_tc_acc, g->d_tc_counter};
-    for (void* p : ptrs)
-        if (p) cudaFree(p);
+    cudaFree(g->w_tc_acc);
     g->w_tc_acc = nullptr;
     g->d_tc_counter = nullptr;
 }
@@ -271,14 +266,14 @@ static cudaError_t launch_backproject_tcs_impl(const mbir_geometry* g, const flo
     auto kern = bf ? (g->tc_bvar ? bwd_tcs_kernel<true, 1> : bwd_tcs_kernel<true, 0>)
                    : (g->tc_bvar ? bwd_tcs_kernel<false, 1> : bwd_tcs_kernel<false, 0>);
     cudaError_t ce = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.smem);
-    if (ce == cudaSuccess) ce = cudaMemsetAsync(g->d_tc_counter, 0, sizeof(int), st);
     if (ce != cudaSuccess) return ce;
     const int ntile = (P.M + kTsTile - 1) / kTsTile;
     const int grid = std::max(1, std::min(g->n_sm, P.K * ntile));
     const void* e = bf ? (const void*)e_bf : (const void*)e_pad;
     const int N = P.W * P.H;
     unsigned int* emax = reinterpret_cast<unsigned int*>(g->w_tc_acc + N);
-    ce = cudaMemsetAsync(g->w_tc_acc, 0, sizeof(unsigned long long) * ((size_t)N + 1), st);
+    // the sums, max |e| and the work counter
+    ce = cudaMemsetAsync(g->w_tc_acc, 0, sizeof(unsigned long long) * ((size_t)N + 2), st);
     if (ce != cudaSuccess) return ce;
     const long long ne = (long long)P.K * P.Mp;
     const int eg = (int)std::max(1LL, std::min((ne + 255) / 256, (long long)g->n_sm * 8));
