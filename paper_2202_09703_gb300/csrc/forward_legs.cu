@@ -8,7 +8,7 @@
 // one run of rows; a cursor per (column, layer) moves on from tile to tile, so each pair is evaluated about
 // once, and none past the record's end.  A tile reaches only one or two layers of a column, so several warps take
 // every nsub-th row of a run each (one thread per run left most threads waiting at the barrier for runs of up to
-// 40 rows: 3.3 ms instead of 2.6).  Nothing is sorted, compacted or staged.
+// 40 rows: 3.3 ms instead of 2.6, before the two forms shared the walk).  Nothing is sorted, compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
 // first one's old value), at a scale that the largest |x| and the number of pixels keep from overflow: exact, so
@@ -17,7 +17,7 @@
 // outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
 // would not (3e-7 against 1.5e-7 from FP64).
 //
-// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.6 ms against 10.7 ms of
+// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.67 ms against 10.7 ms of
 // forward_kernel, which gathers every tap of every pair.  The product takes 0.95 ms of it (its FP32 rate and
 // the shared-memory loads that feed it), the walk over the pairs the rest (latency of the legs and the atomics).
 #include <algorithm>

@@ -44,7 +44,9 @@ __device__ __forceinline__ void finalize_dir(const double* part, int nb, int it,
 // The MAP update and the prior stencil in one pass: with dupd given, x is first moved by the previous
 // iteration's step, x + alpha dupd (alpha = sc[S_ALPHA]), at the pixel and at its eight neighbours, and the
 // moved image is written to xout; then grad = -b/sigma^2 + grad R(x) at the moved image, with FP64 partials
-// of <g,g>, <g,gprev>, <g,dprev>.  Without dupd the image is taken as it is.
+// of <g,g>, <g,gprev>, <g,dprev>.  Without dupd the image is taken as it is.  With hist given, the last block to
+// finish turns the partials into beta (finalize_dir): a launch of one block for that took 5 us, of an
+// iteration's 100 on a 64x64 image (20 iterations there, with the step's launch saved too: 2.01 -> 1.91 ms).
 __global__ void grad_kernel(GeomParams P, PriorParams pr, const float* __restrict__ x, const float* __restrict__ b,
                             const float* __restrict__ msq, const float* __restrict__ gprev,
                             const float* __restrict__ dprev, float* __restrict__ grad, double* __restrict__ part,
