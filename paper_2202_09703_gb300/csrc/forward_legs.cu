@@ -11,7 +11,7 @@
 // 40 rows: 3.3 ms instead of 2.6, before the two forms shared the walk).  Nothing is sorted, compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
-// first one's old value), at a scale that the largest |x| and the number of pixels keep from overflow: exact, so
+// first one's old value), at a scale that the largest |x| and the most pairs of a tile keep from overflow: exact, so
 // the result does not depend on the order of the additions and every output bit is reproducible.  The product
 // with the table is FP32 on the CUDA cores: it is a short convolution per column, which a thread does for four
 // outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     const int R = P.Q + 1, dR = P.G > 1 ? R : 0;
     const int* htx = D.hidx + (size_t)__ldg(D.txpos + k / P.n_rx) * P.W;
     const int* hrx = D.hidx + (size_t)__ldg(D.rxpos + k) * P.W;
-    // fixed-point scale: |x| < 2^ex and weights of at most 1 (2 with rounding), W x H of them, stay below 2^62
+    // fixed-point scale: |x| < 2^ex and weights of at most 1 (2 with rounding), a tile's pairs of them, stay below 2^62
     int ex = 0;
     frexpf(__uint_as_float(__ldg(xmax)), &ex);
     const int se = sbits - ex;
@@ -447,14 +447,15 @@ __global__ void bl_finish_kernel(int N, const unsigned long long* __restrict__ a
 }
 
 // Attenuation planes that the pairs of each (A-scan, tile) reach, as the range of table columns first | end << 16
-// (0: no pair); *wmax: the widest.  Block per A-scan.
+// (0: no pair); wmax: the widest, and the most pairs of a tile.  Block per A-scan.
 __global__ void fl_range_kernel(GeomParams P, DevPtrs D, uint32_t* __restrict__ crange, int* __restrict__ wmax)
 {
-    __shared__ int lo[kFlMaxTiles], hi[kFlMaxTiles];
+    __shared__ int lo[kFlMaxTiles], hi[kFlMaxTiles], count[kFlMaxTiles];
     const int k = blockIdx.x, ntile = (P.M + kFlTile - 1) / kFlTile;
     for (int t = threadIdx.x; t < ntile; t += blockDim.x) {
         lo[t] = 1 << 30;
         hi[t] = -1;
+        count[t] = 0;
     }
     __syncthreads();
     const int tp = __ldg(D.txpos + k / P.n_rx), rp = __ldg(D.rxpos + k);
@@ -468,6 +469,7 @@ __global__ void fl_range_kernel(GeomParams P, DevPtrs D, uint32_t* __restrict__ 
         const int t = pr.n0 / kFlTile;
         if (pr.gi < lo[t]) atomicMin(lo + t, pr.gi);
         if (pr.gi > hi[t]) atomicMax(hi + t, pr.gi);
+        atomicAdd(count + t, 1);
     }
     __syncthreads();
     const int R = P.Q + 1;
@@ -477,6 +479,7 @@ __global__ void fl_range_kernel(GeomParams P, DevPtrs D, uint32_t* __restrict__ 
             const int a = lo[t] * R, b = (min(hi[t] + 1, P.G - 1) + 1) * R;
             r = (uint32_t)a | (uint32_t)b << 16;
             atomicMax(wmax, b - a);
+            atomicMax(wmax + 1, count[t]);
         }
         crange[(size_t)k * ntile + t] = r;
     }
@@ -494,12 +497,12 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
     uint32_t* d_cr = nullptr;
     float* d_tab = nullptr;
     unsigned int* d_max = nullptr;
-    int wmax = 0;
+    int wmax[2] = {0, 0};
     const size_t ncr = (size_t)P.K * ntile, ntab = (size_t)P.G * R * P.Tw4;
     cudaError_t e = cudaMalloc((void**)&d_cr, sizeof(uint32_t) * ncr);
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_tab, sizeof(float) * ntab);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_max, sizeof(unsigned int));
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, sizeof(unsigned int), st);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_max, sizeof(wmax));
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, sizeof(wmax), st);
     if (e == cudaSuccess) {
         bool table = false;
         e = solve_otf_legs(g, st, &table);
@@ -508,7 +511,7 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
         fl_range_kernel<<<P.K, 1024, 0, st>>>(P, dev_ptrs(g), d_cr, reinterpret_cast<int*>(d_max));
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&wmax, d_max, sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(wmax, d_max, sizeof(wmax), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     float tmax = 0.0f, tsum = 0.0f;
     unsigned char* d_acc = nullptr;                  // per pixel: the adjoint's sum, (one word) max |e|, the NaN marks
@@ -532,7 +535,7 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
             }
         e = cudaMemcpy(d_tab, tab.data(), sizeof(float) * ntab, cudaMemcpyHostToDevice);
     }
-    const int kw = std::max(wmax, 1);
+    const int kw = std::max(wmax[0], 1);
     const size_t sm = fl_layout(P, kw).smem;
     if (e == cudaSuccess && sm > 226 * 1024) e = cudaErrorNotSupported;     // a tile reaches too many planes
     if (e == cudaSuccess)
@@ -551,7 +554,7 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
     }
     int np = 0, ext = 0;
-    while ((1LL << np) < (long long)P.W * P.H) ++np;
+    while ((1LL << np) < (long long)wmax[1]) ++np;
     std::frexp(tmax, &ext);
     g->fl_bits = 61 - np;
     g->fl_ebits = std::max(ext, 0);
@@ -561,7 +564,7 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
     g->d_fl_max = d_max;
     g->w_fl_acc = d_acc;
     g->fl_bound = (float)bound;
-    g->bytes += sizeof(uint32_t) * ncr + sizeof(float) * ntab + sizeof(unsigned int) + nacc;
+    g->bytes += sizeof(uint32_t) * ncr + sizeof(float) * ntab + sizeof(wmax) + nacc;
     return cudaSuccess;
 }
 
