@@ -1,8 +1,8 @@
 // A x (eq. 11-13 summed over voxels) as a gather: one CTA per A-scan.  The CTA
 // walks the image in blocks of columns.  For each block it writes one record
 // per (column, row) pair - first tap sample, table row, bilinear weights times
-// x - into shared memory.  Inside one layer the travel time grows with depth,
-// so each (column, layer) segment of records is sorted by first sample; for
+// x - into shared memory.  Among rows that cross the same layers the travel
+// time grows with depth, so each (column, segment of such rows) of records is sorted by first sample; for
 // every 32-sample span of the A-scan the rows whose 68-tap window reaches the
 // span form one contiguous run.  The run bounds of every (segment, span) are
 // written by a conflict-free scatter (each bound is owned by exactly one row),

@@ -4,11 +4,12 @@
 //     y[n0 + 1 + m] += sum_col S[n0][col] T[col][m],       col = plane * (Q + 1) + phase,
 // for one tile of 128 values of n0 after another.
 //
-// Pairs: in one layer the delay grows with depth, so each (column, layer) of the image holds a tile's pixels in
-// one run of rows; a cursor per (column, layer) moves on from tile to tile, so each pair is evaluated about
-// once, and none past the record's end.  A tile reaches only one or two layers of a column, so several warps take
-// every nsub-th row of a run each (one thread per run left most threads waiting at the barrier for runs of up to
-// 40 rows: 3.3 ms instead of 2.6, before the two forms shared the walk).  Nothing is sorted, compacted or staged.
+// Pairs: among rows that cross the same layers (a segment: GeomParams::seg_row) the delay grows with depth, so each
+// (column, segment) of the image holds a tile's pixels in one run of rows; a cursor per (column, segment) moves on
+// from tile to tile, so each pair is evaluated about once, and none past the record's end.  A tile reaches only one
+// or two segments of a column, so several warps take every nsub-th row of a run each (one thread per run left most
+// threads waiting at the barrier for runs of up to 40 rows: 3.3 ms instead of 2.6, before the two forms shared the
+// walk).  Nothing is sorted, compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
 // first one's old value), at a scale that the largest |x| and the most pairs of a tile keep from overflow: exact, so
@@ -94,7 +95,7 @@ __device__ __forceinline__ long long fl_word(unsigned int lo, unsigned int hi)
 
 __device__ __forceinline__ Leg fl_leg(float4 v) { return Leg{v.x, v.y, v.z, v.w}; }
 
-// The cursors at tile t0: the first row of each (layer, column) whose pair starts in that tile or later.  A cursor
+// The cursors at tile t0: the first row of each (segment, column) whose pair starts in that tile or later.  A cursor
 // is row << 16 | its tile (0: not looked at); nxt, for the next tile, starts past each run's end.
 template <int NT>
 __device__ __forceinline__ void fl_cursors(const GeomParams& P, const DevPtrs& D, const int* htx, const int* hrx, int t0,
@@ -117,7 +118,7 @@ __device__ __forceinline__ void fl_cursors(const GeomParams& P, const DevPtrs& D
 }
 
 // Calls pair(row, column, pair, n0 - tile's start, x) for every pair of the tile t (of non-zero weight or not), and
-// sets nxt to the runs' next rows.  A warp takes 32 columns and every nsub-th row of each layer's run, with enough
+// sets nxt to the runs' next rows.  A warp takes 32 columns and every nsub-th row of each segment's run, with enough
 // warps per run for every warp of the block to take part.
 template <int NT, typename F>
 __device__ __forceinline__ void fl_walk(const GeomParams& P, const DevPtrs& D, const int* htx, const int* hrx,

@@ -269,16 +269,19 @@ int mbir_create_geometry(const mbir_geometry_desc* d, void* stream, mbir_geometr
     size_t bytes = 0;
     cudaError_t ce = cudaSuccess;
     std::vector<RowInfo> rows(P.H);
-    int prev_lv = -1;
+    int prev_nl = -1;
     P.n_seg = 0;
     for (int r = 0; r < P.H; ++r) {
         double z = d->img_z0_m + (r + 0.5) * d->pitch_m;
         double eta[MBIR_MAX_LAYERS];
         int nl;
         int lv = layer_of(d, z, eta, &nl);
-        if (lv != prev_lv) {
+        // by the layers crossed: a row on an interface belongs to the layer below, but its delay is that of a path
+        // through the layers above, which past the critical angle is later than the refracted paths of the rows
+        // below it
+        if (nl != prev_nl) {
             P.seg_row[P.n_seg++] = r;
-            prev_lv = lv;
+            prev_nl = nl;
         }
         RowInfo& ri = rows[r];
         ri.nl = nl;

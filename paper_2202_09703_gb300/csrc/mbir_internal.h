@@ -31,7 +31,7 @@ struct GeomParams {
     float2 s2[kMaxLayers];            // (fs / c_l)^2 as double-float
     float2 eta[kMaxLayers];           // full layer thickness as double-float
     float alpha_c[kMaxLayers];        // alpha_l (s/m) * gscale: gamma-bin units per metre
-    int n_seg;                        // layer segments among image rows
+    int n_seg;                        // segments of rows that cross the same layers (delays grow with depth)
     int seg_row[kMaxLayers + 1];      // first row of each segment, seg_row[n_seg] = H
     int apod_first;                   // eq. 12 with the first-layer angle instead of the angle sum
     float2 tilt_c, tilt_s;            // cos / sin of the transmitter firing angle (double-float)
