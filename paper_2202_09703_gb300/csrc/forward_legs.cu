@@ -6,10 +6,12 @@
 //
 // Pairs: among rows that cross the same layers (a segment: GeomParams::seg_row) the delay grows with depth, so each
 // (column, segment) of the image holds a tile's pixels in one run of rows; a cursor per (column, segment) moves on
-// from tile to tile, so each pair is evaluated about once, and none past the record's end.  A tile reaches only one
-// or two segments of a column, so several warps take every nsub-th row of a run each (one thread per run left most
-// threads waiting at the barrier for runs of up to 40 rows: 3.3 ms instead of 2.6, before the two forms shared the
-// walk).  Nothing is sorted, compacted or staged.
+// from tile to tile, so each pair is evaluated about once, and none past the record's end.  Just below an interface
+// the delay of steep pairs grows by less per row than its rounding error (1e-5 of it at most, under one sample), so
+// every bound of a run leaves one sample for pairs out of order.  A tile reaches only one or two segments of a column,
+// so several warps take every nsub-th row of a run each (one thread per run left most threads waiting at the barrier
+// for runs of up to 40 rows: 3.3 ms instead of 2.6, before the two forms shared the walk).  Nothing is sorted,
+// compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
 // first one's old value), at a scale that the largest |x| and the most pairs of a tile keep from overflow: exact, so
@@ -95,8 +97,9 @@ __device__ __forceinline__ long long fl_word(unsigned int lo, unsigned int hi)
 
 __device__ __forceinline__ Leg fl_leg(float4 v) { return Leg{v.x, v.y, v.z, v.w}; }
 
-// The cursors at tile t0: the first row of each (segment, column) whose pair starts in that tile or later.  A cursor
-// is row << 16 | its tile (0: not looked at); nxt, for the next tile, starts past each run's end.
+// The cursors at tile t0: the first row of each (segment, column) whose pair starts in that tile or later, or one
+// sample before it.  A cursor is row << 16 | the first tile that its pair or a later one can start in (0: not looked
+// at); nxt, for the next tile, starts past each run's end.
 template <int NT>
 __device__ __forceinline__ void fl_cursors(const GeomParams& P, const DevPtrs& D, const int* htx, const int* hrx, int t0,
                                            unsigned int* cur, unsigned int* nxt)
@@ -109,7 +112,7 @@ __device__ __forceinline__ void fl_cursors(const GeomParams& P, const DevPtrs& D
         while (a < b) {
             const int mid = (a + b) >> 1;
             const float4* lr = D.legs + (size_t)mid * P.nh;
-            if (make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)), 1.0f).n0 < t0 * kFlTile) a = mid + 1;
+            if (make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)), 1.0f).n0 < t0 * kFlTile - 1) a = mid + 1;
             else b = mid;
         }
         cur[j] = (unsigned int)a << 16;
@@ -154,12 +157,13 @@ __device__ __forceinline__ void fl_walk(const GeomParams& P, const DevPtrs& D, c
                 }
                 const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
                 const int n0r = pr.n0 - t * kFlTile;
-                if (pr.n0 + 1 >= P.M) break;                       // the rows below start later still
+                if (pr.n0 >= P.M) break;                           // the rows below start at M - 1 or later
                 if (n0r >= kFlTile) {
-                    atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)(pr.n0 / kFlTile));
-                    break;
+                    atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)((pr.n0 - 1) / kFlTile));
+                    if (n0r > kFlTile) break;                      // the rows below start in later tiles
+                } else if (n0r >= 0 && pr.n0 + 1 < P.M && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) {
+                    pair(row, col, pr, n0r, xv);
                 }
-                if (n0r >= 0 && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) pair(row, col, pr, n0r, xv);
                 row += nsub;
                 if (row >= end) break;
                 a = an;
