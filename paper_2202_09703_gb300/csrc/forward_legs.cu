@@ -14,13 +14,15 @@
 // compacted or staged.
 //
 // S is summed in 64-bit fixed point in shared memory (two 32-bit atomics per corner, the carry taken from the
-// first one's old value), at a scale that the largest |x| and the most pairs of a tile keep from overflow: exact, so
-// the result does not depend on the order of the additions and every output bit is reproducible.  The product
+// first one's old value), at a scale that the largest |x| and the tile's largest weight and number of pairs keep from
+// overflow: exact, so the result does not depend on the order of the additions and every output bit is reproducible.
+// A tile none of whose sums has kFlMinBits bits at that scale (x there is far below its largest) is walked again at the
+// scale of its largest |w x|: the grid stays finer than FP32 beside the tile's own sums.  The product
 // with the table is FP32 on the CUDA cores: it is a short convolution per column, which a thread does for four
 // outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
 // would not (3e-7 against 1.5e-7 from FP64).
 //
-// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.67 ms against 10.7 ms of
+// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.63 ms against 10.7 ms of
 // forward_kernel, which gathers every tap of every pair.  The product takes 0.95 ms of it (its FP32 rate and
 // the shared-memory loads that feed it), the walk over the pairs the rest (latency of the legs and the atomics).
 #include <algorithm>
@@ -34,6 +36,7 @@ namespace mbir {
 constexpr int kFlTile = 128;                     // values of n0 per tile
 constexpr int kFlThreads = 1024;
 constexpr int kFlMaxTiles = 512;                 // tiles of an A-scan (set-up's shared memory)
+constexpr int kFlMinBits = 30;                   // of a tile's largest sum on its fixed-point grid
 
 // Shared memory: S as low and high words (columns of 128), then the edge taps' words, the share sums, carries,
 // row flags and cursors.
@@ -129,6 +132,7 @@ __device__ __forceinline__ void fl_walk(const GeomParams& P, const DevPtrs& D, c
                                         F&& pair)
 {
     const int ngrp = (P.W + 31) / 32, nsub = min(16, max(1, NT / 32 / ngrp)), units = ngrp * nsub;
+    const int lim = min(kFlTile, P.M - 1 - t * kFlTile);           // past the tile's, and the record's, last n0
     for (int u = threadIdx.x >> 5; u < units; u += NT / 32) {
         const int sub = u / ngrp, col = (u - sub * ngrp) * 32 + (threadIdx.x & 31);
         if (col >= P.W) continue;
@@ -144,31 +148,27 @@ __device__ __forceinline__ void fl_walk(const GeomParams& P, const DevPtrs& D, c
             if (row >= end) continue;
             const float4* lr = D.legs + (size_t)row * P.nh;
             float4 a = __ldg(lr + ht), b = __ldg(lr + hr);
-            float xv = x ? __ldg(x + (size_t)row * P.W + col) : 0.0f;
             for (;;) {
                 // the next row's legs load while this one's pair is evaluated
                 lr += (size_t)nsub * P.nh;
                 float4 an = a, bn = b;
-                float xn = 0.0f;
+                const float xv = x ? __ldg(x + (size_t)row * P.W + col) : 0.0f;
                 if (row + nsub < end) {
                     an = __ldg(lr + ht);
                     bn = __ldg(lr + hr);
-                    if (x) xn = __ldg(x + (size_t)(row + nsub) * P.W + col);
                 }
                 const Pair pr = make_pair(P, fl_leg(a), fl_leg(b), __ldg(&D.rows[row].tau));
                 const int n0r = pr.n0 - t * kFlTile;
-                if (pr.n0 >= P.M) break;                           // the rows below start at M - 1 or later
-                if (n0r >= kFlTile) {
-                    atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)((pr.n0 - 1) / kFlTile));
-                    if (n0r > kFlTile) break;                      // the rows below start in later tiles
-                } else if (n0r >= 0 && pr.n0 + 1 < P.M && __ldg(&D.rows[row].tvert) < (float)(P.M - 1)) {
-                    pair(row, col, pr, n0r, xv);
+                if (n0r > lim) {                                   // the rows below start in later tiles
+                    atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)((min(pr.n0, P.M) - 1) / kFlTile));
+                    break;
                 }
+                if (n0r == lim) atomicMin(nxt + j, (unsigned int)row << 16 | (unsigned int)t);
+                if ((unsigned)n0r < (unsigned)lim) pair(row, col, pr, n0r, xv);
                 row += nsub;
                 if (row >= end) break;
                 a = an;
                 b = bn;
-                xv = xn;
             }
         }
     }
@@ -186,8 +186,8 @@ __device__ __forceinline__ void fl_advance(const GeomParams& P, unsigned int*& c
 
 // Block (A-scan, chunk of tiles): tiles [ta, tb), and the one before for the taps that reach past it.
 __global__ void __launch_bounds__(kFlThreads, 1)
-    forward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint32_t* __restrict__ crange,
-                        const float* __restrict__ x, const unsigned int* __restrict__ xmax, int sbits, int ebits,
+    forward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint2* __restrict__ crange,
+                        const float* __restrict__ x, const unsigned int* __restrict__ xmax, int ebits,
                         int kwmax, int per, float* __restrict__ y_f32, __nv_bfloat16* __restrict__ y_bf16,
                         int out_stride)
 {
@@ -198,6 +198,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     float* part = reinterpret_cast<float*>(smem + L.off_part);
     float* carry = reinterpret_cast<float*>(smem + L.off_carry);
     int* bad = reinterpret_cast<int*>(smem + L.off_bad);                 // rows with a non-finite x; [128]: any
+    unsigned int* smax = reinterpret_cast<unsigned int*>(bad + kFlTile + 1);    // bits of the tile's largest |S|, |w x|
     // cursors of this tile and of the next, per (layer, column)
     unsigned int* cur = reinterpret_cast<unsigned int*>(smem + L.off_cur);
     unsigned int* nxt = cur + (size_t)P.W * P.n_seg;
@@ -208,10 +209,8 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     const int R = P.Q + 1, dR = P.G > 1 ? R : 0;
     const int* htx = D.hidx + (size_t)__ldg(D.txpos + k / P.n_rx) * P.W;
     const int* hrx = D.hidx + (size_t)__ldg(D.rxpos + k) * P.W;
-    // fixed-point scale: |x| < 2^ex and weights of at most 1 (2 with rounding), a tile's pairs of them, stay below 2^62
-    int ex = 0;
+    int ex = 0;                                                          // |x| < 2^ex
     frexpf(__uint_as_float(__ldg(xmax)), &ex);
-    const int se = sbits - ex;
 
     auto store = [&](int n, float v) {
         if (y_f32) y_f32[(size_t)k * out_stride + n] = v;
@@ -219,7 +218,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     };
     for (size_t i = tid; i < L.off_part / 4; i += kFlThreads) lo[i] = 0u;
     if (tid < 2 * kFlTile) carry[tid] = 0.0f;
-    if (tid <= kFlTile) bad[tid] = 0;
+    if (tid <= kFlTile + 2) bad[tid] = 0;
     if (ta == 0 && tid == 0) store(0, 0.0f);
     if (tb == ntile)
         for (int n = P.M + tid; n < out_stride; n += kFlThreads) store(n, 0.0f);
@@ -230,9 +229,14 @@ __global__ void __launch_bounds__(kFlThreads, 1)
     int par = 0;
     for (int t = t0; t < tb; ++t) {
         const int ts = t * kFlTile;
-        const uint32_t cr = __ldg(crange + (size_t)k * ntile + t);
-        const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
-        if (kw > 0) {
+        const uint2 cr = __ldg(crange + (size_t)k * ntile + t);
+        const int c_lo = (int)(cr.x & 0xffffu), kw = (int)(cr.x >> 16) - c_lo;
+        // fixed-point scale: weights below 2^(cr.y >> 16), |x| below 2^ex and the tile's pairs of them stay below 2^61
+        // (2^62 with the rounding of the products)
+        const int nbits = (int)(cr.y & 0xffffu);
+        int se = min(nbits - ((int)cr.y >> 16) - ex, 250);
+        bool rescaled = false;
+        for (bool again = kw > 0; again;) {
             // ---- the tile's pairs into S
             fl_walk<kFlThreads>(P, D, htx, hrx, x, t, cur, nxt, [&](int row, int col, const Pair& pr, int n0r, float xv) {
                 const float wx = pr.w * xv;
@@ -262,15 +266,52 @@ __global__ void __launch_bounds__(kFlThreads, 1)
             // ---- S as FP32 in place of its low words
             uint4* l4 = reinterpret_cast<uint4*>(lo);
             uint4* h4 = reinterpret_cast<uint4*>(lo + hiw);
+            float sm = 0.0f;
             for (int i = tid; i < kw * (kFlTile / 4); i += kFlThreads) {
                 const uint4 l = l4[i], h = h4[i];
                 h4[i] = make_uint4(0u, 0u, 0u, 0u);
-                l4[i] = make_uint4(__float_as_uint(fl_scale(__ll2float_rn(fl_word(l.x, h.x)), -se)),
-                                   __float_as_uint(fl_scale(__ll2float_rn(fl_word(l.y, h.y)), -se)),
-                                   __float_as_uint(fl_scale(__ll2float_rn(fl_word(l.z, h.z)), -se)),
-                                   __float_as_uint(fl_scale(__ll2float_rn(fl_word(l.w, h.w)), -se)));
+                const float4 v = make_float4(__ll2float_rn(fl_word(l.x, h.x)), __ll2float_rn(fl_word(l.y, h.y)),
+                                             __ll2float_rn(fl_word(l.z, h.z)), __ll2float_rn(fl_word(l.w, h.w)));
+                sm = fmaxf(fmaxf(sm, fmaxf(fabsf(v.x), fabsf(v.y))), fmaxf(fabsf(v.z), fabsf(v.w)));
+                l4[i] = make_uint4(__float_as_uint(fl_scale(v.x, -se)), __float_as_uint(fl_scale(v.y, -se)),
+                                   __float_as_uint(fl_scale(v.z, -se)), __float_as_uint(fl_scale(v.w, -se)));
             }
+            unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(sm));
+            if ((tid & 31) == 0 && m) atomicMax(smax, m);
             __syncthreads();
+            again = !rescaled && __uint_as_float(*smax) < (float)(1u << kFlMinBits) && __ldg(xmax) != 0;
+            if (again) {
+                // too coarse a grid, unless the sums are small by cancellation: the tile's largest |w x|
+                m = 0;
+                for (int j = tid; j < P.W * P.n_seg; j += kFlThreads) {
+                    const int sg = j / P.W, col = j - sg * P.W;
+                    const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
+                    for (int row = (int)(cur[j] >> 16); row < P.seg_row[sg + 1]; ++row) {
+                        const float4* lr = D.legs + (size_t)row * P.nh;
+                        const Pair pr = make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)),
+                                                  __ldg(&D.rows[row].tau));
+                        const int n0r = pr.n0 - ts;
+                        if (n0r > kFlTile) break;
+                        const unsigned int b = __float_as_uint(pr.w * __ldg(x + (size_t)row * P.W + col)) & 0x7fffffffu;
+                        if (n0r >= 0 && n0r < kFlTile && pr.n0 + 1 < P.M && b < 0x7f800000u) m = max(m, b);
+                    }
+                }
+                m = __reduce_max_sync(0xffffffffu, m);
+                if ((tid & 31) == 0 && m) atomicMax(smax + 1, m);
+                __syncthreads();
+                int em = 0;
+                frexpf(__uint_as_float(smax[1]), &em);
+                rescaled = true;
+                again = smax[1] != 0 && em + se < kFlMinBits;
+                if (again) {
+                    se = nbits - em;
+                    for (int i = tid; i < kw * (kFlTile / 4); i += kFlThreads) l4[i] = make_uint4(0u, 0u, 0u, 0u);
+                    if (tid < 2 * kFlTile) edge[tid] = 0u;
+                    __syncthreads();
+                }
+            }
+        }
+        if (kw > 0) {
             // ---- outputs 4 og .. 4 og + 3 of this thread's columns: sum_m S[o - m] T[m], four taps at a time
             // against the blocks of four values of S at and below the output
             if (cg < L.ncg) {
@@ -331,53 +372,65 @@ __global__ void __launch_bounds__(kFlThreads, 1)
         __syncthreads();
         if (kw > 0) {
             if (tid < 2 * kFlTile) edge[tid] = 0u;
-            if (tid <= kFlTile) bad[tid] = 0;
+            if (tid <= kFlTile + 2) bad[tid] = 0;
             __syncthreads();
         }
     }
 }
 
 constexpr int kBlThreads = 512;
+// The A^T's sums are kept on two grids: a tile whose residual is below 2^-kBlFiner of the largest adds to a grid that
+// much finer, so that its pairs keep FP32's bits down to 2^-2 kBlFiner of the largest residual.
+constexpr int kBlFiner = 25;
 
 struct BlLayout {
-    size_t off_e, off_cur, smem;
+    size_t off_e, off_max, off_cur, smem;
 };
 __host__ __device__ inline BlLayout bl_layout(const GeomParams& P, int kw)
 {
     BlLayout L;
     L.off_e = (size_t)kw * kFlTile * 4;
-    L.off_cur = L.off_e + (size_t)(kFlTile + P.Tw4) * 4;
+    L.off_max = L.off_e + (size_t)(kFlTile + P.Tw4) * 4;
+    L.off_cur = L.off_max + 16;
     L.smem = L.off_cur + (((size_t)P.W * P.n_seg * 8 + 15) & ~(size_t)15);
     return L;
 }
 
-// Scale exponent of the adjoint's fixed-point sums: every contribution is at most bound / K x max |e| in magnitude
-// and a pixel has at most one per A-scan, so no partial sum reaches 2^61.
-__device__ __forceinline__ int bl_exponent(unsigned int emax_bits, float bound)
+// Scale of the adjoint's fixed-point sums: 2^bl_exponent times the pixel's own power of two (FlPlanes, fl_unit_kernel).
+// Every contribution is at most max |e| / (2 K unit) in magnitude and a pixel has at most one per A-scan, so with the
+// rounding of the products no partial sum reaches 2^61.
+__device__ __forceinline__ int bl_exponent(unsigned int emax_bits)
 {
-    int e1 = 0, e2 = 0;
-    frexpf(__uint_as_float(emax_bits), &e1);
-    frexpf(bound, &e2);
-    return 61 - e1 - e2;
+    int ex = 0;
+    frexpf(__uint_as_float(emax_bits), &ex);
+    return 61 - ex;
 }
+
+// Per attenuation plane: the largest sum of |T| over a table row, plus the largest |T| (the tau = t0 tap).
+struct FlPlanes {
+    float b[64];
+};
 
 // A^T r from the legs, the adjoint of the sums above: for a tile of 128 values of n0
 //     C[n0][col] = sum_m e[n0 + 1 + m] T[col][m]
 // (FP32, eight values of n0 and a share of the columns per thread), of which each pair combines four, and adds the
-// result to its pixel's 64-bit fixed-point sum.  Block (A-scan, chunk of tiles), two blocks per SM: one's products
+// result to its pixel's 64-bit fixed-point sum, in units of the largest that one of the pixel's pairs can add (so that
+// a pixel far from every transducer is summed on as fine a grid, relative to its value, as one below them; one unit and
+// one grid for the image took 1.26 ms and lost pixels of weights below 1e-13 altogether).  Block (A-scan, chunk of tiles), two blocks per SM: one's products
 // run beside the other's walk.
-// 256x512, 64 x 16 A-scans (41 M pairs, FP32), legs included: 1.25 ms against 2.26 ms of backproject_kernel, which
+// 256x512, 64 x 16 A-scans (41 M pairs, FP32), legs included: 1.29 ms against 2.26 ms of backproject_kernel, which
 // is bound by the shared-memory loads of its taps (83 % of their peak); the walk takes about half of it.
 template <typename E>
 __global__ void __launch_bounds__(kBlThreads, 2)
-    backward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint32_t* __restrict__ crange,
-                         const E* __restrict__ e, const unsigned int* __restrict__ emax, float bound, int kwmax, int per,
-                         unsigned long long* __restrict__ acc, unsigned char* __restrict__ bad)
+    backward_legs_kernel(GeomParams P, DevPtrs D, const float* __restrict__ ftab, const uint2* __restrict__ crange,
+                         const E* __restrict__ e, const unsigned int* __restrict__ emax, const unsigned char* __restrict__ unit,
+                         int kwmax, int per, unsigned long long* __restrict__ acc, unsigned char* __restrict__ bad)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     const BlLayout L = bl_layout(P, kwmax);
     float* C = reinterpret_cast<float*>(smem);
     float* sE = reinterpret_cast<float*>(smem + L.off_e);
+    unsigned int* smax = reinterpret_cast<unsigned int*>(smem + L.off_max);    // bits of max |e| of this and the next tile
     unsigned int* cur = reinterpret_cast<unsigned int*>(smem + L.off_cur);
     unsigned int* nxt = cur + (size_t)P.W * P.n_seg;
     const int tid = threadIdx.x, k = blockIdx.x;
@@ -386,18 +439,32 @@ __global__ void __launch_bounds__(kBlThreads, 2)
     const int R = P.Q + 1, dR = P.G > 1 ? R : 0;
     const int* htx = D.hidx + (size_t)__ldg(D.txpos + k / P.n_rx) * P.W;
     const int* hrx = D.hidx + (size_t)__ldg(D.rxpos + k) * P.W;
-    const int se = bl_exponent(__ldg(emax), bound);
+    const int se0 = bl_exponent(__ldg(emax));
     const int cg = tid >> 4, og = tid & 15;
+    if (tid < 2) smax[tid] = 0u;
     fl_cursors<kBlThreads>(P, D, htx, hrx, ta, cur, nxt);
+    __syncthreads();
+    int par = 0;
     for (int t = ta; t < tb; ++t) {
-        const uint32_t cr = __ldg(crange + (size_t)k * ntile + t);
+        const uint32_t cr = __ldg(&crange[(size_t)k * ntile + t].x);
         const int c_lo = (int)(cr & 0xffffu), kw = (int)(cr >> 16) - c_lo;
         if (kw <= 0) continue;
+        unsigned int em = 0;
         for (int i = tid; i < kFlTile + P.Tw4; i += kBlThreads) {
             const int n = t * kFlTile + 1 + i;
-            sE[i] = n < P.Mp ? fl_float(e[(size_t)k * P.Mp + n]) : 0.0f;
+            const float v = n < P.Mp ? fl_float(e[(size_t)k * P.Mp + n]) : 0.0f;
+            sE[i] = v;
+            const unsigned int b = __float_as_uint(v) & 0x7fffffffu;
+            if (b < 0x7f800000u) em = max(em, b);
         }
+        em = __reduce_max_sync(0xffffffffu, em);
+        if ((tid & 31) == 0 && em) atomicMax(smax + par, em);
         __syncthreads();
+        const bool fine = bl_exponent(smax[par]) - kBlFiner >= se0;
+        const int se = se0 + (fine ? kBlFiner : 0);
+        unsigned long long* const sum = acc + (fine ? (size_t)P.W * P.H : 0);
+        par ^= 1;
+        if (tid == 0) smax[par] = 0u;                              // (two barriers before the next tile's)
         // ---- C, rows 8 og .. 8 og + 7: four taps at a time against the window's next four samples
         const float4* W = reinterpret_cast<const float4*>(sE);
         const int ntb = P.Tw4 / 4;
@@ -423,6 +490,8 @@ __global__ void __launch_bounds__(kBlThreads, 2)
         __syncthreads();
         fl_walk<kBlThreads>(P, D, htx, hrx, nullptr, t, cur, nxt, [&](int row, int col, const Pair& pr, int n0r, float) {
             if (pr.w == 0.0f) return;
+            const int px = row * P.W + col;
+            const float u = __uint_as_float((unsigned int)__ldg(unit + px) << 23);
             const float* c = C + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
             const float p1 = pr.psi, p0 = 1.0f - pr.psi;
             float hv = pr.w0 * (p0 * c[0] + p1 * c[dR * kFlTile]) +
@@ -433,34 +502,52 @@ __global__ void __launch_bounds__(kBlThreads, 2)
                 hv -= pr.w1 * (p0 * __ldg(tl) + p1 * __ldg(tl + dR * P.Tw4)) * sE[n0r + P.Tw - 1];
             }
             const float v = pr.w * hv;
-            const int px = row * P.W + col;
-            if (fabsf(v) <= 3.4028235e38f) red_add_global_u64(acc + px, (unsigned long long)__float2ll_rn(fl_scale(v, se)));
-            else bad[px] = 1;
+            if (fabsf(v) <= 3.4028235e38f)
+                red_add_global_u64(sum + px, (unsigned long long)__float2ll_rn(fl_scale(v, se) * u));
+            else
+                bad[px] = 1;
         });
         __syncthreads();
         fl_advance<kBlThreads>(P, cur, nxt);
     }
 }
 
-// b from the fixed-point sums; NaN where a contribution was not finite
+// b from the fixed-point sums of the two grids; NaN where a contribution was not finite
 __global__ void bl_finish_kernel(int N, const unsigned long long* __restrict__ acc, const unsigned char* __restrict__ bad,
-                                 const unsigned int* __restrict__ emax, float bound, float* __restrict__ b)
+                                 const unsigned int* __restrict__ emax, const unsigned char* __restrict__ unit,
+                                 float* __restrict__ b)
 {
-    const int se = bl_exponent(*emax, bound);
+    const int se = bl_exponent(*emax);
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x)
-        b[v] = bad[v] ? __uint_as_float(0x7fc00000u) : fl_scale(__ll2float_rn((long long)acc[v]), -se);
+        b[v] = bad[v] ? __uint_as_float(0x7fc00000u) : fl_scale((float)((double)(long long)acc[v] + (double)(long long)acc[N + v] / (1 << kBlFiner)) /
+                                                              __uint_as_float((unsigned int)unit[v] << 23), -se);
 }
 
-// Attenuation planes that the pairs of each (A-scan, tile) reach, as the range of table columns first | end << 16
-// (0: no pair); wmax: the widest, and the most pairs of a tile.  Block per A-scan.
-__global__ void fl_range_kernel(GeomParams P, DevPtrs D, uint32_t* __restrict__ crange, int* __restrict__ wmax)
+// unit[v] = biased exponent of 2^-e for bounds[v] 2 K < 2^e (bounds[v]: bits of the largest contribution of one of the
+// pixel's pairs at max |e| = 1, 0 for none)
+__global__ void fl_unit_kernel(int N, int K, const unsigned int* __restrict__ bounds, unsigned char* __restrict__ unit)
+{
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < N; v += gridDim.x * blockDim.x) {
+        int e = 0;
+        frexpf(__uint_as_float(bounds[v]) * (2.0f * (float)K), &e);
+        unit[v] = (unsigned char)(min(max(-e, -120), 120) + 127);
+    }
+}
+
+// Per (A-scan, tile): x = the attenuation planes that its pairs reach, as the range of table columns first | end << 16
+// (0: no pair), y = the bits that their number leaves of 61 | exponent of the largest weight << 16; wide: the widest
+// range; bounds: for fl_unit_kernel (zero before).  Block per A-scan.
+__global__ void fl_range_kernel(GeomParams P, DevPtrs D, FlPlanes planes, uint2* __restrict__ crange,
+                                int* __restrict__ wide, unsigned int* __restrict__ bounds)
 {
     __shared__ int lo[kFlMaxTiles], hi[kFlMaxTiles], count[kFlMaxTiles];
+    __shared__ unsigned int wmax[kFlMaxTiles];
     const int k = blockIdx.x, ntile = (P.M + kFlTile - 1) / kFlTile;
     for (int t = threadIdx.x; t < ntile; t += blockDim.x) {
         lo[t] = 1 << 30;
         hi[t] = -1;
         count[t] = 0;
+        wmax[t] = 0;
     }
     __syncthreads();
     const int tp = __ldg(D.txpos + k / P.n_rx), rp = __ldg(D.rxpos + k);
@@ -475,16 +562,22 @@ __global__ void fl_range_kernel(GeomParams P, DevPtrs D, uint32_t* __restrict__ 
         if (pr.gi < lo[t]) atomicMin(lo + t, pr.gi);
         if (pr.gi > hi[t]) atomicMax(hi + t, pr.gi);
         atomicAdd(count + t, 1);
+        const unsigned int wb = __float_as_uint(fabsf(pr.w));
+        if (wb > wmax[t]) atomicMax(wmax + t, wb);
+        const unsigned int cb = __float_as_uint(fabsf(pr.w) * fmaxf(planes.b[pr.gi], planes.b[min(pr.gi + 1, P.G - 1)]));
+        if (cb > *(volatile unsigned int*)(bounds + v)) atomicMax(bounds + v, cb);
     }
     __syncthreads();
     const int R = P.Q + 1;
     for (int t = threadIdx.x; t < ntile; t += blockDim.x) {
-        uint32_t r = 0;
+        uint2 r = make_uint2(0u, 0u);
         if (hi[t] >= 0) {
             const int a = lo[t] * R, b = (min(hi[t] + 1, P.G - 1) + 1) * R;
-            r = (uint32_t)a | (uint32_t)b << 16;
-            atomicMax(wmax, b - a);
-            atomicMax(wmax + 1, count[t]);
+            int ew = 0;
+            frexpf(__uint_as_float(wmax[t]), &ew);
+            const int np = 32 - __clz(count[t] - 1);            // count <= 2^np
+            r = make_uint2((uint32_t)a | (uint32_t)b << 16, (uint32_t)(61 - np) | (uint32_t)ew << 16);
+            atomicMax(wide, b - a);
         }
         crange[(size_t)k * ntile + t] = r;
     }
@@ -499,78 +592,93 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
     if (!g->d_legs || g->d_rec_key || g->d_tf4_bop || P.Tw > kFlTile || ntile > kFlMaxTiles || P.G * R > 65535 ||
         P.H > 65535 || (long long)P.W * P.n_seg > 8192)
         return cudaErrorNotSupported;
-    uint32_t* d_cr = nullptr;
+    // the table by columns, its largest value and the planes' bounds
+    const bool bf = P.precision == MBIR_PREC_BF16;
+    const int nq = P.Q * P.Tw + 1;
+    const size_t ncr = (size_t)P.K * ntile, ntab = (size_t)P.G * R * P.Tw4, N = (size_t)P.W * P.H;
+    std::vector<float> tab(ntab, 0.0f);
+    FlPlanes planes{};
+    float tmax = 0.0f, bmax = 0.0f;
+    for (int gp = 0; gp < P.G; ++gp) {
+        float pmax = 0.0f, psum = 0.0f;
+        for (int r = 0; r < R; ++r) {
+            float sum = 0.0f;
+            for (int m = 0; m < P.Tw; ++m) {
+                float v = (float)g->tab_host[(size_t)gp * nq + m * P.Q + r];
+                if (bf) v = __bfloat162float(__float2bfloat16_rn(v));
+                tab[((size_t)gp * R + r) * P.Tw4 + m] = v;
+                pmax = std::max(pmax, std::fabs(v));
+                sum += std::fabs(v);
+            }
+            psum = std::max(psum, sum);
+        }
+        planes.b[gp] = psum + pmax;
+        tmax = std::max(tmax, pmax);
+        bmax = std::max(bmax, planes.b[gp]);
+    }
+    if (!(bmax > 0.0f && bmax < 1e12f)) return cudaErrorNotSupported;        // (keeps the scaled sums in range)
+    uint2* d_cr = nullptr;
     float* d_tab = nullptr;
-    unsigned int* d_max = nullptr;
-    int wmax[2] = {0, 0};
-    const size_t ncr = (size_t)P.K * ntile, ntab = (size_t)P.G * R * P.Tw4;
-    cudaError_t e = cudaMalloc((void**)&d_cr, sizeof(uint32_t) * ncr);
+    unsigned int *d_max = nullptr, *d_bound = nullptr;
+    unsigned char* d_unit = nullptr;
+    unsigned char* d_acc = nullptr;                  // per pixel: the adjoint's sums, (one word) max |e|, the NaN marks
+    const size_t nacc = 17 * N + 8;
+    int wide = 0;
+    cudaError_t e = cudaMalloc((void**)&d_cr, sizeof(uint2) * ncr);
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_tab, sizeof(float) * ntab);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_max, sizeof(wmax));
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, sizeof(wmax), st);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_max, sizeof(wide));
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_unit, N);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_bound, sizeof(unsigned int) * N);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_acc, nacc);
+    if (e == cudaSuccess) e = cudaMemcpy(d_tab, tab.data(), sizeof(float) * ntab, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_max, 0, sizeof(wide), st);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d_bound, 0, sizeof(unsigned int) * N, st);
     if (e == cudaSuccess) {
         bool table = false;
         e = solve_otf_legs(g, st, &table);
     }
     if (e == cudaSuccess) {
-        fl_range_kernel<<<P.K, 1024, 0, st>>>(P, dev_ptrs(g), d_cr, reinterpret_cast<int*>(d_max));
+        fl_range_kernel<<<P.K, 1024, 0, st>>>(P, dev_ptrs(g), planes, d_cr, reinterpret_cast<int*>(d_max), d_bound);
+        fl_unit_kernel<<<(int)std::min<size_t>((N + 255) / 256, 1024), 256, 0, st>>>((int)N, P.K, d_bound, d_unit);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(wmax, d_max, sizeof(wmax), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&wide, d_max, sizeof(wide), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    float tmax = 0.0f, tsum = 0.0f;
-    unsigned char* d_acc = nullptr;                  // per pixel: the adjoint's sum, (one word) max |e|, the NaN marks
-    const size_t nacc = 9 * (size_t)P.W * P.H + 8;
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_acc, nacc);
-    if (e == cudaSuccess) {
-        const bool bf = P.precision == MBIR_PREC_BF16;
-        const int nq = P.Q * P.Tw + 1;
-        std::vector<float> tab(ntab, 0.0f);
-        for (int gp = 0; gp < P.G; ++gp)
-            for (int r = 0; r < R; ++r) {
-                float sum = 0.0f;
-                for (int m = 0; m < P.Tw; ++m) {
-                    float v = (float)g->tab_host[(size_t)gp * nq + m * P.Q + r];
-                    if (bf) v = __bfloat162float(__float2bfloat16_rn(v));
-                    tab[((size_t)gp * R + r) * P.Tw4 + m] = v;
-                    tmax = std::max(tmax, std::fabs(v));
-                    sum += std::fabs(v);
-                }
-                tsum = std::max(tsum, sum);
-            }
-        e = cudaMemcpy(d_tab, tab.data(), sizeof(float) * ntab, cudaMemcpyHostToDevice);
-    }
-    const int kw = std::max(wmax[0], 1);
+    cudaFree(d_bound);
+    const int kw = std::max(wide, 1);
     const size_t sm = fl_layout(P, kw).smem;
     if (e == cudaSuccess && sm > 226 * 1024) e = cudaErrorNotSupported;     // a tile reaches too many planes
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(forward_legs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
     for (const void* f : {(const void*)backward_legs_kernel<float>, (const void*)backward_legs_kernel<__nv_bfloat16>})
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024);
-    // weights are at most 1 (2 with the rounding of the products)
-    const double bound = 2.0 * P.K * ((double)tsum + tmax);
-    if (e == cudaSuccess && !(bound > 0.0 && bound < 1e30)) e = cudaErrorNotSupported;
     if (e != cudaSuccess) {
         cudaFree(d_cr);
         cudaFree(d_tab);
         cudaFree(d_max);
+        cudaFree(d_unit);
         cudaFree(d_acc);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
     }
-    int np = 0, ext = 0;
-    while ((1LL << np) < (long long)wmax[1]) ++np;
+    int ext = 0;
     std::frexp(tmax, &ext);
-    g->fl_bits = 61 - np;
     g->fl_ebits = std::max(ext, 0);
     g->fl_kw = kw;
     g->d_fl_crange = d_cr;
     g->d_fl_tab = d_tab;
     g->d_fl_max = d_max;
     g->w_fl_acc = d_acc;
-    g->fl_bound = (float)bound;
-    g->bytes += sizeof(uint32_t) * ncr + sizeof(float) * ntab + sizeof(wmax) + nacc;
+    g->d_fl_unit = d_unit;
+    g->bytes += sizeof(uint2) * ncr + sizeof(float) * ntab + N + sizeof(wide) + nacc;
     return cudaSuccess;
+}
+
+// Ends the segments at the first row whose vertical path already ends past the record (no pair below it is active).
+static void fl_clip_rows(const mbir_geometry* g, GeomParams& P)
+{
+    const int rows = (int)(std::lower_bound(g->h_tvert, g->h_tvert + P.H, (float)(P.M - 1)) - g->h_tvert);
+    for (int i = 0; i <= P.n_seg; ++i) P.seg_row[i] = std::min(P.seg_row[i], rows);
 }
 
 // One block per A-scan runs alone on its SM, so few A-scans leave SMs idle: their tiles are then cut into chunks
@@ -578,15 +686,16 @@ cudaError_t build_forward_legs(mbir_geometry* g, cudaStream_t st)
 cudaError_t launch_forward_legs(const mbir_geometry* g, const float* x, float* yf, __nv_bfloat16* yb, int stride,
                                 cudaStream_t st)
 {
-    const GeomParams& P = g->P;
+    GeomParams P = g->P;
     const int N = P.W * P.H, ntile = (P.M + kFlTile - 1) / kFlTile;
+    fl_clip_rows(g, P);
     cudaError_t e = cudaMemsetAsync(g->d_fl_max, 0, sizeof(unsigned int), st);
     if (e != cudaSuccess) return e;
     fl_xmax_kernel<float><<<std::max(1, std::min((N + 1023) / 1024, g->n_sm)), 256, 0, st>>>(N, x, g->d_fl_max);
     const int want = (4 * g->n_sm + P.K - 1) / P.K;
     const int per = std::max((ntile + want - 1) / want, std::min(4, ntile));
     forward_legs_kernel<<<dim3(P.K, (ntile + per - 1) / per), kFlThreads, fl_layout(P, g->fl_kw).smem, st>>>(
-        P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, x, g->d_fl_max, g->fl_bits, g->fl_ebits, g->fl_kw, per, yf, yb,
+        P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, x, g->d_fl_max, g->fl_ebits, g->fl_kw, per, yf, yb,
         stride);
     return cudaGetLastError();
 }
@@ -596,12 +705,13 @@ cudaError_t launch_forward_legs(const mbir_geometry* g, const float* x, float* y
 cudaError_t launch_backproject_legs(const mbir_geometry* g, const float* e_pad, const __nv_bfloat16* e_bf, float* b,
                                     cudaStream_t st)
 {
-    const GeomParams& P = g->P;
+    GeomParams P = g->P;
     const int N = P.W * P.H, ntile = (P.M + kFlTile - 1) / kFlTile;
+    fl_clip_rows(g, P);
     auto* acc = reinterpret_cast<unsigned long long*>(g->w_fl_acc);
-    auto* emax = reinterpret_cast<unsigned int*>(acc + N);
-    unsigned char* bad = g->w_fl_acc + 8 * ((size_t)N + 1);
-    cudaError_t e = cudaMemsetAsync(g->w_fl_acc, 0, 9 * (size_t)N + 8, st);
+    auto* emax = reinterpret_cast<unsigned int*>(acc + 2 * (size_t)N);
+    unsigned char* bad = g->w_fl_acc + 8 * (2 * (size_t)N + 1);
+    cudaError_t e = cudaMemsetAsync(g->w_fl_acc, 0, 17 * (size_t)N + 8, st);
     if (e != cudaSuccess) return e;
     const long long ne = (long long)P.K * P.Mp;
     const int eg = (int)std::max(1LL, std::min((ne + 255) / 256, (long long)g->n_sm * 8));
@@ -612,15 +722,16 @@ cudaError_t launch_backproject_legs(const mbir_geometry* g, const float* e_pad, 
     if (P.precision == MBIR_PREC_BF16) {
         fl_xmax_kernel<__nv_bfloat16><<<eg, 256, 0, st>>>(ne, e_bf, emax);
         backward_legs_kernel<__nv_bfloat16><<<grid, kBlThreads, sm, st>>>(
-            P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, e_bf, emax, g->fl_bound, g->fl_kw, per, acc, bad);
+            P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, e_bf, emax, g->d_fl_unit, g->fl_kw, per, acc, bad);
     } else {
         fl_xmax_kernel<float><<<eg, 256, 0, st>>>(ne, e_pad, emax);
         backward_legs_kernel<float><<<grid, kBlThreads, sm, st>>>(
-            P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, e_pad, emax, g->fl_bound, g->fl_kw, per, acc, bad);
+            P, dev_ptrs(g), g->d_fl_tab, g->d_fl_crange, e_pad, emax, g->d_fl_unit, g->fl_kw, per, acc, bad);
     }
     e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    bl_finish_kernel<<<std::max(1, std::min((N + 255) / 256, g->n_sm * 8)), 256, 0, st>>>(N, acc, bad, emax, g->fl_bound, b);
+    bl_finish_kernel<<<std::max(1, std::min((N + 255) / 256, g->n_sm * 8)), 256, 0, st>>>(N, acc, bad, emax, g->d_fl_unit,
+                                                                                            b);
     return cudaGetLastError();
 }
 

@@ -392,14 +392,14 @@ struct mbir_geometry {
     int* d_bwd_counter;    // work counter of the A^T r launch
     float* h_bwd_cost;     // host copy: estimated A^T r cost per (16-row tile, 32-column tile, Tx position)
     int bwd_ntc;           // 32-column tiles per row of tiles
-    // A x without stored records, from the legs (forward_legs.cu): column ranges per (A-scan, tile), the table by
-    // columns, the largest |x| of the call; bits of the fixed-point sums and of the table, widest column range
-    uint32_t* d_fl_crange;
+    // A x without stored records, from the legs (forward_legs.cu): column ranges and bits of the fixed-point sums per
+    // (A-scan, tile), the table by columns, the largest |x| of the call; bits of the table, widest column range
+    uint2* d_fl_crange;
     float* d_fl_tab;
     unsigned int* d_fl_max;
-    int fl_bits, fl_ebits, fl_kw;
-    unsigned char* w_fl_acc;   // the adjoint's workspace (N 64-bit sums, max |e|, N marks) and its scale bound
-    float fl_bound;
+    int fl_ebits, fl_kw;
+    unsigned char* w_fl_acc;   // the adjoint's workspace (2 N 64-bit sums, max |e|, N marks)
+    unsigned char* d_fl_unit;  // and the power of two (biased exponent) that scales each pixel's sum
     // TAB-mode A x records sorted by first tap sample (see forward_tab.cu); with the tensor-core applies the
     // sorted records are replaced by their packed form (tc_apply.cuh), on the same per-A-scan offsets
     long long* d_rec_off;
