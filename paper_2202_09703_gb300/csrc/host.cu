@@ -173,7 +173,7 @@ void free_geometry(mbir_geometry* g)
                     g->d_legs, g->d_hidx, g->d_hvals, g->d_hsign, g->d_fl_crange, g->d_fl_tab, g->d_fl_max, g->w_fl_acc, g->d_fl_unit, g->d_direct, g->d_dinv, g->d_status, g->w_e, g->w_q,
                     g->w_b, g->w_grad, g->w_gprev, g->w_d, g->w_part, g->w_scal, g->w_ebf,
                     g->w_msq, g->w_d2, g->w_xalt, g->w_y, g->w_x, g->w_g, g->w_hist, g->d_items, g->w_bpart,
-                    g->d_rec_off, g->d_rec_key, g->d_rec_w, g->d_tc_key, g->d_tc_w, g->d_runs, g->d_win_order, g->d_win_counter,
+                    g->d_rec_off, g->d_rec_key, g->d_rec_n0, g->d_rec_w, g->d_tc_key, g->d_tc_w, g->d_runs, g->d_win_order, g->d_win_counter,
                     g->d_bwd_counter, g->d_tb_key, g->d_tb_w, g->d_tb_tile, g->w_tc_acc,
                     g->d_tf_order, g->d_tf_counter, g->w_colnorm,
                     g->d_tf4_bop, g->d_tf4_crange, g->d_tf4_split, g->d_tb4_bop, g->d_tf_view, g->d_tb_view};
@@ -561,19 +561,18 @@ int mbir_create_geometry(const mbir_geometry_desc* d, void* stream, mbir_geometr
         if (ce == cudaErrorNotSupported) ce = cudaSuccess;     // keep the on-the-fly record path
         if (ce != cudaSuccess) { free_geometry(g); return cuda_err(ce); }
         if (g->d_rec_key && !(d->flags & MBIR_FLAG_NO_TENSOR_CORES)) {
-            // A x first: it leaves the records in its kernel's order, on which the adjoint's slots are built
             ce = mbir::build_tc_forward_stream(g, st);
             if (ce == cudaErrorNotSupported) ce = cudaSuccess;  // keep the CUDA-core A x
             if (ce != cudaSuccess) { free_geometry(g); return cuda_err(ce); }
             ce = mbir::build_tc_adjoint(g, st);
-            if (ce == cudaErrorNotSupported) ce = cudaSuccess;  // keep the CUDA-core adjoint
-            if (ce != cudaSuccess) { free_geometry(g); return cuda_err(ce); }
-            ce = mbir::build_tc_adjoint_stream(g, st);
+            if (ce == cudaSuccess) ce = mbir::build_tb_records(g, st);
+            if (ce == cudaSuccess) ce = mbir::build_tc_adjoint_stream(g, st);
             if (ce == cudaErrorNotSupported) {                  // keep the CUDA-core A^T
                 mbir::free_tc_adjoint(g);
                 ce = cudaSuccess;
             }
             if (ce != cudaSuccess) { free_geometry(g); return cuda_err(ce); }
+            if (g->d_tf4_bop) mbir::free_sorted_keys(g);
         }
         // the tensor-core pools' variants are chosen by timing them once
         if (g->d_tf4_bop || g->d_tb4_bop) {

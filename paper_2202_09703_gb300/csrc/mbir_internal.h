@@ -404,6 +404,7 @@ struct mbir_geometry {
     // sorted records are replaced by their packed form (tc_apply.cuh), on the same per-A-scan offsets
     long long* d_rec_off;
     int2* d_rec_key;
+    int* d_rec_n0;         // set-up only: first record of every n0, K x (M + 1)
     float4* d_rec_w;
     uint2* d_tc_key;       // packed records: keys
     void* d_tc_w;          // and weights (uint2 in the FP32 form, uint32 in the BF16 form)
@@ -468,6 +469,8 @@ struct mbir_geometry {
 
 namespace mbir {
 // launchers implemented in apply.cu
+cudaError_t build_tb_records(mbir_geometry* g, cudaStream_t st);
+void free_sorted_keys(mbir_geometry* g);
 cudaError_t launch_build_legs(const mbir_geometry* g, const int* d_hsign, const float2* d_hvals, cudaStream_t st);
 cudaError_t solve_otf_legs(const mbir_geometry* g, cudaStream_t st, bool* table);
 cudaError_t load_otf_legs(const mbir_geometry* g);

@@ -1,5 +1,5 @@
-// Tables of the tensor-core A^T (tcs_adjoint_pool, tc_stream.cuh): the per-pixel fixed-point accumulators and the bound
-// that sets their scale, the table operand, and the launch: max |e| of the
+// Tables of the tensor-core A^T (tcs_adjoint_pool, tc_stream.cuh): the
+// per-pixel fixed-point accumulators and the bound that sets their scale, the table operand, and the launch: max |e| of the
 // residual, the pool (one integer addition per record into its pixel's sum),
 // then the sums turned into FP32.  Integer addition is associative, so the
 // result does not depend on which CTA adds what when: it is reproducible bit
@@ -64,28 +64,61 @@ __global__ void tc_finish_kernel(int N, const unsigned long long* __restrict__ a
 }
 
 // *wmax = bits of the largest record weight w (the four bilinear corners are non-negative and sum to w)
-template <bool BF16>
-__global__ void tc_wmax_kernel(TbRecs rec, long long n, unsigned int* __restrict__ wmax)
+template <typename WT>
+__global__ void tc_wmax_kernel(const WT* __restrict__ rw, long long n, unsigned int* __restrict__ wmax)
 {
     unsigned int m = 0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    {
-        TbRec<BF16> r;
-        r.load(rec, (size_t)i);
-        m = max(m, __float_as_uint(fabsf(r.weight())));
-    }
+        m = max(m, __float_as_uint(fabsf(tc_rec_w(rw[i]))));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0 && m) atomicMax(wmax, m);
 }
 
-// The per-pixel accumulators (N sums and the max |e| word after them, zeroed) and the bound of the fixed-point scale: K x the largest record weight w x (the largest table row sum
-// of |T| + the largest |T|, for the tau = t0 tap), doubled for the rounding of the products;
-// cudaErrorNotSupported keeps the CUDA-core adjoint.
+Tb4Layout tb4_layout(const GeomParams& P, int kwmax)
+{
+    Tb4Layout L{};
+    const bool bf = P.precision == MBIR_PREC_BF16;
+    L.parts = bf ? 1 : 2;
+    L.R = P.Q + 1;
+    L.kb = (P.G * L.R + 15) & ~15;
+    L.ntap = (P.Tw + 15) & ~15;
+    L.kwmax = std::min(std::min(kwmax, 256), L.kb);
+    L.cstride = ((L.kwmax + 31) & ~31) + 4;            // 4 mod 32: the read-back rows hit distinct banks
+    L.ewin = (kTsTile + L.ntap + 31) & ~31;
+    L.bbytes = (size_t)L.parts * L.kb * L.ntap * 2;
+    L.off_e = 256;                                     // after the header and the warps' maxima
+    L.off_b = (L.off_e + (size_t)2 * L.ewin * 4 + 1023) & ~(size_t)1023;
+    L.off_c = (L.off_b + L.bbytes + 1023) & ~(size_t)1023;
+    L.smem = L.off_c + (size_t)kTsTile * L.cstride * 4;
+    L.ok = L.R >= 2 && L.ntap <= 128 && L.kwmax >= 16 && L.kwmax % 16 == 0 && 128 + L.kwmax <= (int)kTsCols &&
+           kTsTile + L.ntap <= 32 * tb_warps(bf) && L.smem <= 227 * 1024 && L.bbytes < (1u << 20) &&
+           P.G * L.R <= 4096;
+    return L;
+}
+
+// The layout for the widest tile of a geometry whose A x is set up; false when the A^T does not fit the tensor cores.
+static bool tb4_choose(const mbir_geometry* g, Tb4Layout* out)
+{
+    const GeomParams& P = g->P;
+    Tb4Layout L{};
+    for (int kw : {256, 224, 192, 160, 128, 96, 64}) {
+        L = tb4_layout(P, kw);
+        if (L.ok) break;
+    }
+    if (!L.ok || g->tf4_wmax > L.kwmax) return false;
+    const Tb4Layout Lt = tb4_layout(P, std::max(g->tf4_wmax, 16));           // no wider than the widest tile
+    *out = Lt.ok ? Lt : L;
+    return true;
+}
+
+// The per-pixel accumulators (N sums, the max |e| word and the work counter, zeroed) and the bound of the fixed-point
+// scale: K x the largest record weight w x (the largest table row sum of |T| + the largest |T|, for the tau = t0 tap),
+// doubled for the rounding of the products; cudaErrorNotSupported keeps the CUDA-core adjoint.
 cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
 {
     const GeomParams& P = g->P;
-    if (!g->d_tb_key || g->n_records <= 0) return cudaErrorNotSupported;
+    if (!g->d_tc_key || g->n_records <= 0) return cudaErrorNotSupported;
     const int N = P.W * P.H;
     unsigned long long* d_acc = nullptr;
     cudaError_t e = cudaMalloc((void**)&d_acc, sizeof(unsigned long long) * ((size_t)N + 2));
@@ -93,11 +126,12 @@ cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
     unsigned int wbits = 0;
     if (e == cudaSuccess) {
         unsigned int* d_wmax = reinterpret_cast<unsigned int*>(d_acc + N);
-        const TbRecs rec{g->d_tb_key, g->d_tb_w};
         if (P.precision == MBIR_PREC_BF16)
-            tc_wmax_kernel<true><<<std::max(1, g->n_sm * 8), 256, 0, st>>>(rec, g->n_records, d_wmax);
+            tc_wmax_kernel<<<std::max(1, g->n_sm * 8), 256, 0, st>>>(reinterpret_cast<const uint32_t*>(g->d_tc_w),
+                                                                     g->n_records, d_wmax);
         else
-            tc_wmax_kernel<false><<<std::max(1, g->n_sm * 8), 256, 0, st>>>(rec, g->n_records, d_wmax);
+            tc_wmax_kernel<<<std::max(1, g->n_sm * 8), 256, 0, st>>>(reinterpret_cast<const uint2*>(g->d_tc_w),
+                                                                     g->n_records, d_wmax);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpyAsync(&wbits, d_wmax, sizeof(wbits), cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(d_wmax, 0, sizeof(unsigned long long), st);
@@ -142,28 +176,6 @@ void free_tc_adjoint(mbir_geometry* g)
 // ---------------------------------------------------------------------------
 // Streamed tensor-core A^T (tcs_adjoint_pool): layout, table operand, launch.
 // ---------------------------------------------------------------------------
-Tb4Layout tb4_layout(const GeomParams& P, int kwmax)
-{
-    Tb4Layout L{};
-    const bool bf = P.precision == MBIR_PREC_BF16;
-    L.parts = bf ? 1 : 2;
-    L.R = P.Q + 1;
-    L.kb = (P.G * L.R + 15) & ~15;
-    L.ntap = (P.Tw + 15) & ~15;
-    L.kwmax = std::min(std::min(kwmax, 256), L.kb);
-    L.cstride = ((L.kwmax + 31) & ~31) + 4;            // 4 mod 32: the read-back rows hit distinct banks
-    L.ewin = (kTsTile + L.ntap + 31) & ~31;
-    L.bbytes = (size_t)L.parts * L.kb * L.ntap * 2;
-    L.off_e = 256;                                     // after the header and the warps' maxima
-    L.off_b = (L.off_e + (size_t)2 * L.ewin * 4 + 1023) & ~(size_t)1023;
-    L.off_c = (L.off_b + L.bbytes + 1023) & ~(size_t)1023;
-    L.smem = L.off_c + (size_t)kTsTile * L.cstride * 4;
-    L.ok = L.R >= 2 && L.ntap <= 128 && L.kwmax >= 16 && L.kwmax % 16 == 0 && 128 + L.kwmax <= (int)kTsCols &&
-           kTsTile + L.ntap <= 32 * tb_warps(bf) && L.smem <= 227 * 1024 && L.bbytes < (1u << 20) &&
-           P.G * L.R <= 4096;
-    return L;
-}
-
 // The view is read from device memory (written at set-up) with the residual as a parameter, as for the
 // tensor-core A x (fwd_tcs_kernel).
 template <bool BF16, int BV>
@@ -192,15 +204,7 @@ cudaError_t build_tc_adjoint_stream(mbir_geometry* g, cudaStream_t st)
     if (!g->d_tb_tile || !g->w_tc_acc || !g->d_tf4_crange || !g->d_tc_counter)
         return cudaErrorNotSupported;
     Tb4Layout L{};
-    for (int kw : {256, 224, 192, 160, 128, 96, 64}) {
-        L = tb4_layout(P, kw);
-        if (L.ok) break;
-    }
-    if (!L.ok || g->tf4_wmax > L.kwmax) return cudaErrorNotSupported;
-    {
-        const Tb4Layout Lt = tb4_layout(P, std::max(g->tf4_wmax, 16));   // no wider than the widest tile
-        if (Lt.ok) L = Lt;
-    }
+    if (!tb4_choose(g, &L)) return cudaErrorNotSupported;
     const int nq = P.Q * P.Tw + 1;
     const size_t part = (size_t)L.kb * L.ntap;
     std::vector<uint16_t> img((size_t)L.parts * part, 0);

@@ -146,6 +146,8 @@ struct TbRec {
 };
 template <bool BF16>
 __host__ __device__ constexpr size_t tb_key_bytes() { return BF16 ? sizeof(uint2) : sizeof(uint4); }
+// bytes of one record in all
+inline size_t tb_record_bytes(bool bf) { return bf ? tb_key_bytes<true>() + sizeof(uint32_t) : tb_key_bytes<false>(); }
 
 // Shared-memory header of the tensor-core kernels: offset 0 the MMA mbarrier, 8 the tensor-memory address,
 // 16 the item slot, 20 the abort flag, 32 the table-copy mbarrier.

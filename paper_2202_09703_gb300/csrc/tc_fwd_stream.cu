@@ -217,7 +217,7 @@ __global__ void ts_batch_flag_kernel(GeomParams P, int R, int nparts, const long
 // records of a warp fell into 28 sectors; the pixels of one image row that a tile reaches lie side by side
 // (64 columns where the delay grows by two samples per column), so in pixel order they fall into about nine.
 // 512x1024 A^T: FP32 7.55 -> 5.83 ms; 256x512 0.478 -> 0.418 ms; 203x331 BF16 0.144 -> 0.128 ms.  It costs a
-// second copy of the packed records.
+// second copy of the packed records (build_tb_records).
 // Block per (A-scan, tile): a bitmap of the tile's pixels, from which each record's place is counted.
 __host__ __device__ inline int tb_map_words(const GeomParams& P) { return ((P.W * P.H + 127) >> 7) << 2; }
 template <bool BF16>
@@ -387,6 +387,8 @@ cudaError_t build_tc_forward_stream(mbir_geometry* g, cudaStream_t st)
     const size_t nrec = (size_t)std::max<long long>(g->n_records, 1);
     uint2* d_key = nullptr;
     void* d_pw = nullptr;
+    TsView* d_view = nullptr;
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_view, sizeof(TsView));
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_key, sizeof(uint2) * nrec);
     if (e == cudaSuccess) e = cudaMalloc(&d_pw, wsz * nrec);
     if (e == cudaSuccess) {
@@ -404,65 +406,28 @@ cudaError_t build_tc_forward_stream(mbir_geometry* g, cudaStream_t st)
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     }
-    // the A^T's copy of the records, where there is memory for it (else the CUDA-core A^T is kept)
-    void* d_tkey = nullptr;
-    uint32_t* d_tpw = nullptr;
-    int* d_toff = nullptr;
-    const size_t tksz = bf ? tb_key_bytes<true>() : tb_key_bytes<false>();
-    if (e == cudaSuccess) {
-        cudaError_t m = cudaMalloc((void**)&d_toff, sizeof(int) * (size_t)P.K * (ntile + 1));
-        if (m == cudaSuccess) m = cudaMalloc(&d_tkey, tksz * nrec);
-        if (m == cudaSuccess && bf) m = cudaMalloc((void**)&d_tpw, sizeof(uint32_t) * nrec);
-        if (m != cudaSuccess) {
-            cudaGetLastError();
-            cudaFree(d_toff);
-            cudaFree(d_tkey);
-            d_toff = nullptr;
-            d_tkey = nullptr;
-            if (m != cudaErrorMemoryAllocation) e = m;
-        }
-    }
-    if (e == cudaSuccess && d_tkey) {
-        auto kern = bf ? tb_pack_kernel<true> : tb_pack_kernel<false>;
-        const size_t sm = (size_t)tb_map_words(P) * 5;
-        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-        if (e == cudaSuccess) {
-            const long long nt = (long long)P.K * (ntile + 1);
-            tb_tile_kernel<<<(int)((nt + 255) / 256), 256, 0, st>>>(P, d_n0, d_toff);
-            kern<<<P.K * ntile, 512, sm, st>>>(P, dev_ptrs(g), g->d_rec_off, d_n0, g->d_rec_key,
-                                              reinterpret_cast<uint2*>(d_tkey), d_tpw);
-            e = cudaGetLastError();
-        }
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    }
     // the kernel's view without the per-call fields
-    TsView* d_view = nullptr;
     if (e == cudaSuccess) {
         const void* tab = bf ? (const void*)g->d_tab_bf16 : (const void*)g->d_tab;
         const TsView V{P, L, d_b, tab, g->d_rec_off, d_cr, d_sp, d_key, d_pw, d_ord, nullptr, nullptr, 0, 0, d_ctr};
-        e = cudaMalloc((void**)&d_view, sizeof(TsView));
-        if (e == cudaSuccess) e = cudaMemcpy(d_view, &V, sizeof(TsView), cudaMemcpyHostToDevice);
+        e = cudaMemcpy(d_view, &V, sizeof(TsView), cudaMemcpyHostToDevice);
     }
     if (e != cudaSuccess) {
-        void* ptrs[] = {d_n0, d_ord, d_ctr, d_cr, d_sp, d_b, d_view, d_key, d_pw, d_toff, d_tkey, d_tpw};
+        void* ptrs[] = {d_n0, d_ord, d_ctr, d_cr, d_sp, d_b, d_view, d_key, d_pw};
         for (void* p : ptrs) cudaFree(p);
         cudaGetLastError();
         return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
     }
-    // the sorted records are not read again (the CUDA-core A x no longer runs for this geometry)
-    cudaFree(g->d_rec_key);
+    // of the sorted records only the keys are read again (by build_tb_records; free_sorted_keys releases them): the
+    // weights go first, so that building the A^T's copy holds no more memory than this function did (FP32 form: 8 + 16
+    // + 16 B per pair after 24 + 16; BF16 form: 8 + 12 + 12 after 24 + 12)
     cudaFree(g->d_rec_w);
-    g->d_rec_key = nullptr;
     g->d_rec_w = nullptr;
+    g->d_rec_n0 = d_n0;
     g->bytes -= (sizeof(int2) + sizeof(float4)) * nrec;
     g->bytes += (sizeof(uint2) + wsz) * nrec;
     g->d_tc_key = d_key;
     g->d_tc_w = d_pw;
-    g->d_tb_key = d_tkey;
-    g->d_tb_w = d_tpw;
-    g->d_tb_tile = d_toff;
-    if (d_tkey) g->bytes += (tksz + (bf ? sizeof(uint32_t) : 0)) * nrec + sizeof(int) * (size_t)P.K * (ntile + 1);
-    cudaFree(d_n0);
     g->d_tf_view = d_view;
     g->tf4 = L;
     g->d_tf_order = d_ord;
@@ -473,6 +438,61 @@ cudaError_t build_tc_forward_stream(mbir_geometry* g, cudaStream_t st)
     g->tf4_wmax = wmax;
     g->bytes += L.bbytes + sizeof(int) * ((size_t)P.K + 1) + sizeof(int) * (size_t)P.K * ntile * (nw + 2);
     return cudaSuccess;
+}
+
+// The A^T's copy of the records, for a geometry whose A x has its own (build_tc_forward_stream): where there is memory
+// for it and for the workspace of a reconstruction after it; else cudaErrorNotSupported keeps the CUDA-core A^T.
+cudaError_t build_tb_records(mbir_geometry* g, cudaStream_t st)
+{
+    const GeomParams& P = g->P;
+    if (!g->d_rec_key || !g->d_rec_n0 || g->n_records <= 0) return cudaErrorNotSupported;
+    const bool bf = P.precision == MBIR_PREC_BF16;
+    const int ntile = (P.M + kTsTile - 1) / kTsTile;
+    const size_t nrec = (size_t)g->n_records, ntoff = (size_t)P.K * (ntile + 1);
+    const size_t copy = tb_record_bytes(bf) * nrec + sizeof(int) * ntoff;
+    const size_t work = sizeof(float) * (5 * (size_t)P.K * P.Mp + 16 * (size_t)P.W * P.H);
+    size_t freeb = 0, totalb = 0;
+    cudaError_t e = cudaMemGetInfo(&freeb, &totalb);
+    if (e != cudaSuccess) return e;
+    if (freeb < copy || freeb + sizeof(int2) * nrec < copy + work) return cudaErrorNotSupported;
+    void* d_key = nullptr;
+    uint32_t* d_w = nullptr;
+    int* d_off = nullptr;
+    e = cudaMalloc((void**)&d_off, sizeof(int) * ntoff);
+    if (e == cudaSuccess) e = cudaMalloc(&d_key, (bf ? tb_key_bytes<true>() : tb_key_bytes<false>()) * nrec);
+    if (e == cudaSuccess && bf) e = cudaMalloc((void**)&d_w, sizeof(uint32_t) * nrec);
+    auto kern = bf ? tb_pack_kernel<true> : tb_pack_kernel<false>;
+    const size_t sm = (size_t)tb_map_words(P) * 5;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    if (e == cudaSuccess) {
+        tb_tile_kernel<<<(int)((ntoff + 255) / 256), 256, 0, st>>>(P, g->d_rec_n0, d_off);
+        kern<<<P.K * ntile, 512, sm, st>>>(P, dev_ptrs(g), g->d_rec_off, g->d_rec_n0, g->d_rec_key,
+                                          reinterpret_cast<uint2*>(d_key), d_w);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) {
+        cudaFree(d_off);
+        cudaFree(d_key);
+        cudaFree(d_w);
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? cudaErrorNotSupported : e;
+    }
+    g->d_tb_key = d_key;
+    g->d_tb_w = d_w;
+    g->d_tb_tile = d_off;
+    g->bytes += copy;
+    return cudaSuccess;
+}
+
+// The sorted records' keys and offsets, which only the set-up of the tensor-core applies reads once A x has its own
+// records.
+void free_sorted_keys(mbir_geometry* g)
+{
+    cudaFree(g->d_rec_key);
+    cudaFree(g->d_rec_n0);
+    g->d_rec_key = nullptr;
+    g->d_rec_n0 = nullptr;
 }
 
 cudaError_t launch_forward_tcs(const mbir_geometry* g, const float* x, float* yf, __nv_bfloat16* yb, int stride,
