@@ -118,7 +118,8 @@ static bool tb4_choose(const mbir_geometry* g, Tb4Layout* out)
 cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
 {
     const GeomParams& P = g->P;
-    if (!g->d_tc_key || g->n_records <= 0) return cudaErrorNotSupported;
+    Tb4Layout L{};
+    if (!g->d_tc_key || g->n_records <= 0 || !tb4_choose(g, &L)) return cudaErrorNotSupported;
     const int N = P.W * P.H;
     unsigned long long* d_acc = nullptr;
     cudaError_t e = cudaMalloc((void**)&d_acc, sizeof(unsigned long long) * ((size_t)N + 2));
@@ -165,12 +166,23 @@ cudaError_t build_tc_adjoint(mbir_geometry* g, cudaStream_t st)
     return cudaSuccess;
 }
 
-// The tables above, freed when the tensor-core A^T is not used after all.
+// The tables above and the A^T's records (build_tb_records), freed when the tensor-core A^T is not used after all.
 void free_tc_adjoint(mbir_geometry* g)
 {
+    const GeomParams& P = g->P;
+    if (g->w_tc_acc) g->bytes -= sizeof(unsigned long long) * ((size_t)P.W * P.H + 2);
+    if (g->d_tb_key)
+        g->bytes -= tb_record_bytes(P.precision == MBIR_PREC_BF16) * (size_t)g->n_records +
+                    sizeof(int) * (size_t)P.K * ((P.M + kTsTile - 1) / kTsTile + 1);
     cudaFree(g->w_tc_acc);
+    cudaFree(g->d_tb_key);
+    cudaFree(g->d_tb_w);
+    cudaFree(g->d_tb_tile);
     g->w_tc_acc = nullptr;
     g->d_tc_counter = nullptr;
+    g->d_tb_key = nullptr;
+    g->d_tb_w = nullptr;
+    g->d_tb_tile = nullptr;
 }
 
 // ---------------------------------------------------------------------------

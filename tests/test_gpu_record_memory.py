@@ -1,6 +1,7 @@
 """Device memory of the two packed record lists of the tensor-core applies (needs a GB300)."""
 import pytest
 
+from oracle import oracle as O
 from paper_2202_09703_gb300 import synth as S
 
 torch = pytest.importorskip("torch")
@@ -15,6 +16,18 @@ B.build()
 from paper_2202_09703_gb300 import mbir as M  # noqa: E402
 
 DEV = torch.device("cuda:0")
+
+
+def test_no_second_list_for_a_cuda_core_adjoint():
+    """A tile of the BF16 form that reaches more than 256 table columns keeps A x on the tensor cores and A^T off
+    them: the geometry then holds one packed list (12 B per pair) where the CUDA-core forms hold 24 B."""
+    s = S.small_scene(n_layers=3, w=64, h=64, n_tx=32, n_rx=16, M=512, name="tiny_planes").copy(precision="bf16")
+    s = s.copy(gamma_max=O.Geometry(s).gamma_max() / 16)
+    tc, cc = M.Geometry(s, mode="tab"), M.Geometry(s, mode="tab", tensor_cores=False)
+    n = tc.info.n_records
+    assert tc.info.forward_tensor_cores and not tc.info.adjoint_tensor_cores
+    assert n == cc.info.n_records and n > 400000
+    assert cc.info.device_bytes - tc.info.device_bytes > 6 * n
 
 
 @pytest.mark.parametrize("precision,per_pair", [("fp32", 51), ("bf16", 49)])
