@@ -121,11 +121,25 @@ typedef struct {
  * grouped by first tap sample (the system matrix of Section 3) so that A x
  * and A^T stream them: 24 bytes per active pair for the CUDA-core kernels,
  * packed to 16 (FP32 form) or 12 bytes (BF16 form) for the tensor-core ones,
- * of which A x and A^T each hold a copy in their own order (without memory
- * for the second copy A^T runs on the CUDA cores);
- * this flag keeps the on-the-fly record path of A x instead (less memory,
- * slower). */
+ * of which A x and A^T each hold a copy in their own order (32 and 24 bytes
+ * per pair in all; while the geometry is created 40 and 36).  Records are kept
+ * where 24 bytes per pair are at most half the free memory and 64 GB; A^T has
+ * no copy, and runs on the CUDA cores, where it would leave less free memory
+ * than a reconstruction's workspace takes or where a tile reaches too many
+ * attenuation planes for the tensor cores.
+ * This flag keeps no records: both applies then run from the table of legs, as
+ * the on-the-fly form does from its workspace (less memory, slower). */
 #define MBIR_FLAG_NO_RECORDS 1
+
+/* Without records (this flag, the on-the-fly form, or no memory for them), with
+ * the legs in a table or workspace, both applies go over tiles of 128 first-tap
+ * samples with sums in 64-bit fixed point and FP32 products: the tile's own
+ * largest values set the grid of A x, the pixel's own largest weight and the
+ * tile's residual that of A^T, so that small values beside large ones keep
+ * FP32's relative accuracy (down to about 2^-50 of max |e| in A^T).  A pixel or
+ * sample that is not finite gives NaN in the samples, or pixels, that it
+ * reaches to within a few samples, and in no other.  Geometries with more than 64 MB of legs, or with
+ * tiles of too many attenuation planes, are applied in FP32 pair by pair. */
 
 /* With records, A and A^T normally run on the tensor cores (both storage
  * forms).  Every tap of a pair shares one table phase (eq. 13 with the
@@ -264,8 +278,9 @@ int mbir_backproject(const mbir_geometry* g, const void* r_dev, float* x_dev, vo
  *     needed, but all calls share the one array: calls whose work overlaps on
  *     the GPU (other streams, other host threads) race and must be
  *     serialised by the caller.  The call also uses the geometry's adjoint
- *     work counter, so it must not overlap any other call that applies A^T
- *     with the same geometry (mbir_backproject, the reconstructions, an
+ *     work counter and, in the on-the-fly form, its leg workspace, so it must
+ *     not overlap any other call that applies A^T (there: or A) with the same
+ *     geometry (mbir_backproject, mbir_forward, the reconstructions, an
  *     engine running a request of that geometry).
  * r_dev: K x M floats; x_dev: N floats, overwritten.  Asynchronous on
  * `stream`; no device memory is allocated or freed. */
