@@ -36,7 +36,7 @@ namespace mbir {
 constexpr int kFlTile = 128;                     // values of n0 per tile
 constexpr int kFlThreads = 1024;
 constexpr int kFlMaxTiles = 512;                 // tiles of an A-scan (set-up's shared memory)
-constexpr int kFlMinBits = 30;                   // of a tile's largest sum on its fixed-point grid
+constexpr int kFlMinBits = 26;                   // of a tile's largest sum on its fixed-point grid
 
 // Shared memory: S as low and high words (columns of 128), then the edge taps' words, the share sums, carries,
 // row flags and cursors.
@@ -238,6 +238,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
         bool rescaled = false;
         for (bool again = kw > 0; again;) {
             // ---- the tile's pairs into S
+            bool any = false;
             fl_walk<kFlThreads>(P, D, htx, hrx, x, t, cur, nxt, [&](int row, int col, const Pair& pr, int n0r, float xv) {
                 const float wx = pr.w * xv;
                 if (!(wx != 0.0f)) return;
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
                     bad[kFlTile] = 1;
                     return;
                 }
+                any = true;
                 const float p1 = pr.psi, p0 = 1.0f - pr.psi;
                 unsigned int* s = lo + (size_t)(pr.gi * R + pr.r - c_lo) * kFlTile + n0r;
                 const float wa = wx * pr.w0, wb = wx * pr.w1;
@@ -262,7 +264,7 @@ __global__ void __launch_bounds__(kFlThreads, 1)
                     fl_add(edge + n0r, kFlTile, __float2ll_rn(fl_scale(ev, se - ebits)));
                 }
             });
-            __syncthreads();
+            any = __syncthreads_or(any);
             // ---- S as FP32 in place of its low words
             uint4* l4 = reinterpret_cast<uint4*>(lo);
             uint4* h4 = reinterpret_cast<uint4*>(lo + hiw);
@@ -279,23 +281,14 @@ __global__ void __launch_bounds__(kFlThreads, 1)
             unsigned int m = __reduce_max_sync(0xffffffffu, __float_as_uint(sm));
             if ((tid & 31) == 0 && m) atomicMax(smax, m);
             __syncthreads();
-            again = !rescaled && __uint_as_float(*smax) < (float)(1u << kFlMinBits) && __ldg(xmax) != 0;
+            again = any && !rescaled && __uint_as_float(*smax) < (float)(1u << kFlMinBits);
             if (again) {
                 // too coarse a grid, unless the sums are small by cancellation: the tile's largest |w x|
                 m = 0;
-                for (int j = tid; j < P.W * P.n_seg; j += kFlThreads) {
-                    const int sg = j / P.W, col = j - sg * P.W;
-                    const int ht = __ldg(htx + col), hr = __ldg(hrx + col);
-                    for (int row = (int)(cur[j] >> 16); row < P.seg_row[sg + 1]; ++row) {
-                        const float4* lr = D.legs + (size_t)row * P.nh;
-                        const Pair pr = make_pair(P, fl_leg(__ldg(lr + ht)), fl_leg(__ldg(lr + hr)),
-                                                  __ldg(&D.rows[row].tau));
-                        const int n0r = pr.n0 - ts;
-                        if (n0r > kFlTile) break;
-                        const unsigned int b = __float_as_uint(pr.w * __ldg(x + (size_t)row * P.W + col)) & 0x7fffffffu;
-                        if (n0r >= 0 && n0r < kFlTile && pr.n0 + 1 < P.M && b < 0x7f800000u) m = max(m, b);
-                    }
-                }
+                fl_walk<kFlThreads>(P, D, htx, hrx, x, t, cur, nxt, [&](int, int, const Pair& pr, int, float xv) {
+                    const unsigned int b = __float_as_uint(pr.w * xv) & 0x7fffffffu;
+                    if (b < 0x7f800000u) m = max(m, b);
+                });
                 m = __reduce_max_sync(0xffffffffu, m);
                 if ((tid & 31) == 0 && m) atomicMax(smax + 1, m);
                 __syncthreads();
