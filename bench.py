@@ -529,7 +529,7 @@ def run_extras(args, M, S, torch, np, scene, geo, y, sigma, x_true, x_fp32, flus
     go = M.Geometry(s1, mode="otf")
     fo, bo = apply_times(torch, go, s1, dev)
     ex["cfg1_otf"] = {"apply_ms": {"forward": fo, "backproject": bo},
-                      "note": "travel times solved in registers on every apply (eq. 4-6); no records"}
+                      "note": "travel times solved on every apply, each distinct leg once (eq. 4-6); no records"}
     go.close()
     torch.cuda.empty_cache()
     if args.served_requests > 0:

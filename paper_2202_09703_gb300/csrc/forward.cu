@@ -2,15 +2,15 @@
 // walks the image in blocks of columns.  For each block it writes one record
 // per (column, row) pair - first tap sample, table row, bilinear weights times
 // x - into shared memory.  Among rows that cross the same layers the travel
-// time grows with depth, so each (column, segment of such rows) of records is sorted by first sample; for
-// every 32-sample span of the A-scan the rows whose 68-tap window reaches the
-// span form one contiguous run.  The run bounds of every (segment, span) are
-// written by a conflict-free scatter (each bound is owned by exactly one row),
-// then each warp produces its spans with counted loops over those runs.
-// Every output sample is owned by one lane: no atomics, a fixed summation
-// order, bitwise reproducible results.  Serves the geometries without stored
-// records that forward_legs.cu does not take (no leg table, or a tile that
-// reaches too many attenuation planes).
+// time grows with depth, so each (column, segment of such rows) of records is
+// sorted by first sample; for every 32-sample span of the A-scan the rows whose
+// 68-tap window reaches the span form one contiguous run.  The run bounds of
+// every (segment, span) are written by a conflict-free scatter (each bound is
+// owned by exactly one row), then each warp produces its spans with counted
+// loops over those runs.  Every output sample is owned by one lane: no atomics,
+// a fixed summation order, bitwise reproducible results.  Serves the geometries
+// without stored records that forward_legs.cu does not take (no leg table, or a
+// tile that reaches too many attenuation planes).
 #include <algorithm>
 
 #include "device_common.cuh"

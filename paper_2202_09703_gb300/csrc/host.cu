@@ -1,6 +1,7 @@
 // Host side of the library: argument validation, the pulse table (built once
 // in FP64 by FFT), per-row and per-transducer tables, device uploads, the
-// leg table of TAB mode (of OTF mode: its list of offsets and workspace), and the C ABI entry points that manage handles.
+// leg table of TAB mode (of OTF mode: its list of offsets and workspace), and
+// the C ABI entry points that manage handles.
 #include <algorithm>
 #include <cmath>
 #include <complex>
@@ -170,7 +171,8 @@ void free_geometry(mbir_geometry* g)
 {
     if (!g) return;
     void* ptrs[] = {g->d_rows, g->d_colx, g->d_pos, g->d_txpos, g->d_rxpos, g->d_tab, g->d_tab_bf16,
-                    g->d_legs, g->d_hidx, g->d_hvals, g->d_hsign, g->d_fl_crange, g->d_fl_tab, g->d_fl_max, g->w_fl_acc, g->d_fl_unit, g->d_direct, g->d_dinv, g->d_status, g->w_e, g->w_q,
+                    g->d_legs, g->d_hidx, g->d_hvals, g->d_hsign, g->d_fl_crange, g->d_fl_tab, g->d_fl_max, g->w_fl_acc,
+                    g->d_fl_unit, g->d_direct, g->d_dinv, g->d_status, g->w_e, g->w_q,
                     g->w_b, g->w_grad, g->w_gprev, g->w_d, g->w_part, g->w_scal, g->w_ebf,
                     g->w_msq, g->w_d2, g->w_xalt, g->w_y, g->w_x, g->w_g, g->w_hist, g->d_items, g->w_bpart,
                     g->d_rec_off, g->d_rec_key, g->d_rec_n0, g->d_rec_w, g->d_tc_key, g->d_tc_w, g->d_runs, g->d_win_order, g->d_win_counter,

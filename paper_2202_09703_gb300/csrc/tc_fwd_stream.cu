@@ -211,11 +211,12 @@ __global__ void ts_batch_flag_kernel(GeomParams P, int R, int nparts, const long
     }
 }
 
-// The records of the A^T, every tile's in pixel order.  The A^T is bound by its per-pixel reductions in the L2,
-// which takes a sector (four pixels' sums) per reduction: 206 G/s where every lane meets another sector, 330,
-// 505 and 630 G/s for runs of 2, 4 and 8 neighbouring pixels.  In the A x's order (by n0, for its sums) the 32
-// records of a warp fell into 28 sectors; the pixels of one image row that a tile reaches lie side by side
-// (64 columns where the delay grows by two samples per column), so in pixel order they fall into about nine.
+// The records of the A^T, every tile's in pixel order.  The A^T is bound by its per-pixel reductions in the L2, which
+// takes a sector (four pixels' sums) at a time: a probe of 64-bit reductions alone ran at 197 G/s where every lane of a
+// warp meets another sector, 392, 520 and 728 G/s for runs of 2, 4 and 8 neighbouring pixels.  In the A x's order (by
+// n0, for its sums) the 32 records of a warp fell into 27 sectors (256x512: 35.4 M for 1.29 M requests); the pixels of
+// one image row that a tile reaches lie side by side (64 columns where the delay grows by two samples per column), so
+// in pixel order they fall into nine (12.0 M).
 // 512x1024 A^T: FP32 7.55 -> 5.83 ms; 256x512 0.478 -> 0.418 ms; 203x331 BF16 0.144 -> 0.128 ms.  It costs a
 // second copy of the packed records (build_tb_records).
 // Block per (A-scan, tile): a bitmap of the tile's pixels, from which each record's place is counted.

@@ -523,8 +523,9 @@ __device__ __forceinline__ bool tcs_forward_pool(const TsView& V, unsigned char*
 // is one matrix product of the residual's Hankel tile H[n][m] = e[ts + 1 + n + m]
 // (128 x taps, in tensor memory as the A operand) and the table rows the tile's
 // records reach (one column range, the B operand resident in shared memory);
-// each record (a tile's are stored in pixel order, tb_pack_kernel) then combines four values of C with its bilinear weights (less
-// the tau = t0 tap of flagged records) into one contribution v and adds it to
+// each record (a tile's are stored in pixel order, tb_pack_kernel) then
+// combines four values of C with its bilinear weights (less the tau = t0 tap
+// of flagged records) into one contribution v and adds it to
 // its pixel's 64-bit fixed-point accumulator: round(v 2^s) by an integer atomic
 // (one scale 2^s per apply, tc_fixed_exponent), so the sum is exact and its
 // value does not depend on the order of the additions; a last kernel turns the
