@@ -22,7 +22,7 @@
 // outputs and a share of the columns, and it keeps FP32's accuracy, which two FP16 parts on the tensor cores
 // would not (3e-7 against 1.5e-7 from FP64).
 //
-// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.63 ms against 10.7 ms of
+// 256x512, 64 x 16 A-scans of 2048 samples (41 M pairs, FP32), legs included: 2.65 ms against 10.7 ms of
 // forward_kernel, which gathers every tap of every pair.  The product takes 0.95 ms of it (its FP32 rate and
 // the shared-memory loads that feed it), the walk over the pairs the rest (latency of the legs and the atomics).
 #include <algorithm>
